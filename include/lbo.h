@@ -55,7 +55,12 @@ typedef enum {
 } lbo_status;
 
 typedef enum {
-  LBO_PREC_FP64 = 0,     /* FP64 transforms and products (the plain path)   */
+  LBO_PREC_FP64 = 0,     /* the FP64 path.  Default kernels: FP64 inputs,
+                            Maxwellians, ratio and combination, transforms
+                            and products of numbers with 64 bits and a common
+                            exponent per block (at least as accurate as FP64
+                            transforms); LBO_OPT_KERNEL 1 and 2: FP64
+                            throughout                                      */
   LBO_PREC_FP32 = 1,     /* FP32 transforms and products, FP64 in/out,
                             FP64 Maxwellians, cut-off and final combination */
   LBO_PREC_FP32X2 = 2,   /* transforms and products in pairs of FP32 numbers
@@ -89,12 +94,12 @@ typedef enum {
   LBO_OPT_HEMISPHERE_P = 6,/* hemisphere rule order p: M = 2 p^2 points (4)   */
   LBO_OPT_PRECISION = 7,   /* lbo_precision                                   */
   LBO_OPT_KERNEL = 8,      /* 0: fastest built kernel set for (N, precision)
-                              (default), 1: the generic plane/axis kernels,
-                              2: the generic kernels with every transform a
-                              two-stage shared-memory FFT (FP64 at N = 32
-                              otherwise runs the hot kernels of L and of
-                              Q(f,f) with one thread per pencil in
-                              registers)                                      */
+                              (default; FP64: fixed point on the integer pipe),
+                              1: the generic plane/axis kernels (FP64 at N = 32
+                              runs the hot ones of L and of Q(f,f) with one
+                              thread per pencil in registers), 2: the generic
+                              kernels with every transform a two-stage
+                              shared-memory FFT                               */
   LBO_OPT_JGROUPS = 9,     /* radial nodes per CTA of the fused FP32 kernel are
                               J / jgroups; 0 (default): chosen from the batch */
   LBO_OPT_Q_SINC_QUADRATURE = 10, /* Q(f,f) only.  1: the loss multiplier
@@ -104,9 +109,9 @@ typedef enum {
                               second mass fix of Sec. 2.3 (Eq. (2.16)): Q^_0
                               vanishes up to rounding.  Takes the generic
                               kernels (also for FP32 at N = 32); 0: off   */
-  LBO_OPT_PLANES = 11      /* planes per CTA of the FP64 register plane kernel
-                              at N = 32 (2, 4 or 8; 0: default, 4): the tile
-                              shape lbo_plan_autotune picks for FP64        */
+  LBO_OPT_PLANES = 11      /* planes per CTA of the FP64 plane kernel of the gain
+                              loop at N = 32 (2, 4 or 8; 0: default, 4): the
+                              tile shape lbo_plan_autotune picks for FP64   */
 } lbo_option;
 
 /* Create a plan for N^3 grids on [-box, box]^3, VHS exponent vhs_omega in

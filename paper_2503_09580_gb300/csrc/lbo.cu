@@ -13,6 +13,7 @@
 
 #include "../../include/lbo.h"
 #include "lbo_internal.h"
+#include "lin_fx.h"
 #include "lin_generic.cuh"
 
 namespace lbo {
@@ -80,6 +81,7 @@ template <typename T, int N>
 static lbo_status build_phit(lbo_plan* p, const double* d_stab, T* d_phit);
 
 static void free_tables(lbo_plan* p) {
+  free_fx_tables(p);
   free_twofold_tables(p);
   void* ptrs[] = {p->d_phi64, p->d_omega64, p->d_phit64, p->d_phi32, p->d_omega32, p->d_phit32, p->d_dummy_params,
                   p->d_dct64, p->d_dct32};
@@ -291,9 +293,12 @@ static lbo_status dispatch_lin(lbo_plan* p, const double* params, const double* 
   return dispatch_generic<T>(p, plain_tables<T>(p), params, g, out, B, p->ws, cuh ? &mc : nullptr);
 }
 
-// kernel set of an apply call: 1 the fused FP32 kernels (N = 32), 0 generic
+// kernel set of an apply call: 1 the fused FP32 kernels (N = 32), 2 FP64 in
+// fixed point on the integer pipe, 0 generic
 static int kernel_path(const lbo_plan* p) {
-  return p->precision == LBO_PREC_FP32 && p->N == 32 && p->kernel_choice == 0 ? 1 : 0;
+  if (p->kernel_choice != 0) return 0;
+  if (p->precision == LBO_PREC_FP64) return 2;
+  return p->precision == LBO_PREC_FP32 && p->N == 32 ? 1 : 0;
 }
 
 // bytes of one real number of the generic path's transform arithmetic
@@ -438,7 +443,8 @@ lbo_status lbo_apply_linearized(lbo_plan* p, const double* params, const double*
     lbo_status st = build_tables(p);
     if (st != LBO_OK) return st;
   }
-  lbo_status st = ensure_workspace(p, batch);
+  const int path = kernel_path(p);
+  lbo_status st = path == 2 ? LBO_OK : ensure_workspace(p, batch);
   if (st != LBO_OK) return st;
   const size_t n3 = (size_t)p->N * p->N * p->N;
   const bool dev = is_device_ptr(params) && is_device_ptr(g) && is_device_ptr(out);
@@ -456,7 +462,6 @@ lbo_status lbo_apply_linearized(lbo_plan* p, const double* params, const double*
     dout = p->stage_out;
   }
   // the Maxwellian cache, if it was made for exactly this call's Maxwellians
-  const int path = kernel_path(p);
   const bool cached = p->mc_valid && p->mc_params == dp && p->mc_batch == batch && p->mc_precision == p->precision &&
                       p->mc_path == path;
   const void* cuh = cached ? p->mc_uh : nullptr;
@@ -470,6 +475,8 @@ lbo_status lbo_apply_linearized(lbo_plan* p, const double* params, const double*
     if (st == LBO_OK && (p->mass_fix || p->moment_fix))
       st = launch_fixes(p, dout, batch, p->N, 2.0 * p->L / p->N, p->stream, &launches);
     p->last_launches = launches;
+  } else if (path == 2) {
+    st = run_linearized_fx(p, dp, dg, dout, batch, cached);
   } else if (is_twofold_precision(p->precision)) {
     st = run_linearized_twofold(p, dp, dg, dout, batch, cuh, cw);
   } else if (is_split16_precision(p->precision)) {
@@ -525,7 +532,8 @@ lbo_status lbo_plan_cache_maxwellians(lbo_plan* p, const double* params, int bat
   const int path = kernel_path(p);
   const size_t N = p->N, HC = N / 2 + 1, n3 = N * N * N;
   const size_t rb = transform_real_bytes(p->precision);
-  const size_t uh_bytes = path == 1 ? fused32_uhat_bytes(batch, p->J) : (size_t)p->J * batch * HC * HC * HC * rb;
+  const size_t uh_bytes = path == 1 ? fused32_uhat_bytes(batch, p->J)
+                          : path == 2 ? fx_cache_bytes(p, batch) : (size_t)p->J * batch * HC * HC * HC * rb;
   const size_t w_bytes = path == 1 ? 0 : (size_t)batch * n3 * rb;
   auto grow = [&](void*& ptr, size_t& cap, size_t need) -> lbo_status {
     if (need <= cap) return LBO_OK;
@@ -545,6 +553,7 @@ lbo_status lbo_plan_cache_maxwellians(lbo_plan* p, const double* params, int bat
   if (st == LBO_OK && path == 0) st = ensure_workspace(p, batch);
   if (st != LBO_OK) return st;
   if (path == 1) st = precompute_fused32(p, params, batch, (float*)p->mc_uh);
+  else if (path == 2) st = precompute_fx(p, params, batch);
   else if (is_twofold_precision(p->precision)) st = precompute_twofold(p, params, batch, p->mc_uh, p->mc_w);
   else if (p->precision == LBO_PREC_FP64)
     st = dispatch_precompute<double>(p, plain_tables<double>(p), params, batch, p->ws, p->mc_uh, p->mc_w);

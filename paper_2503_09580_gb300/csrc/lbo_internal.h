@@ -37,6 +37,8 @@ struct lbo_plan {
   void* d_wbf[2] = {nullptr, nullptr};
   void* d_wfp[2] = {nullptr, nullptr};
   void* d_tc_err = nullptr;
+  void* d_fx = nullptr;  // multipliers of the fixed-point form of FP64 (lin_fx_plan.cu)
+  int fx_omega_exp = 0;
   void* tc_scratch = nullptr;
   size_t tc_scratch_bytes = 0;
   // reductions of the slab-block primitives (slab_block.cu)

@@ -91,6 +91,17 @@ __device__ __forceinline__ void fill_maxwellian_tables(double* em, double* thr, 
   __syncthreads();
 }
 
+// The smallest |v-u|^2 for which fl(|v-u|^2 / (2 theta)) > thr, thr =
+// ln(1/eps) - 1.5 ln(2 pi theta) (see fill_ratio_tables).
+__device__ __forceinline__ double cut_distance(double theta, double log_inv_eps) {
+  const double twoth = __dmul_rn(2.0, theta);
+  const double thr = __dsub_rn(log_inv_eps, __dmul_rn(1.5, log(__dmul_rn(__dmul_rn(2.0, 3.141592653589793), theta))));
+  double x = __dmul_rn(thr, twoth);
+  for (int it = 0; it < 64 && __ddiv_rn(x, twoth) > thr; ++it) x = nextafter(x, -1e308);
+  for (int it = 0; it < 64 && !(__ddiv_rn(x, twoth) > thr); ++it) x = nextafter(x, 1e308);
+  return x;
+}
+
 // Tables of the ratio source r = g/M, filled once per CTA:
 //   ei[d*N + i] = exp(+(v_i - u_d)^2 / (2 theta)), axis 0 divided by the
 //   prefactor rho (2 pi theta)^{-3/2}, so 1/M = ei[i1] ei[N+i2] ei[2N+i3];
@@ -109,14 +120,7 @@ __device__ __forceinline__ void fill_ratio_tables(double* ei, double* dstar, con
     if (d == 0) e /= q.rho * pow(2.0 * 3.141592653589793 * q.theta, -1.5);
     ei[t] = e;
   }
-  if (threadIdx.x == 0) {
-    const double twoth = __dmul_rn(2.0, q.theta);
-    const double thr = __dsub_rn(log_inv_eps, __dmul_rn(1.5, log(__dmul_rn(__dmul_rn(2.0, 3.141592653589793), q.theta))));
-    double x = __dmul_rn(thr, twoth);
-    for (int it = 0; it < 64 && __ddiv_rn(x, twoth) > thr; ++it) x = nextafter(x, -1e308);
-    for (int it = 0; it < 64 && !(__ddiv_rn(x, twoth) > thr); ++it) x = nextafter(x, 1e308);
-    *dstar = x;
-  }
+  if (threadIdx.x == 0) *dstar = cut_distance(q.theta, log_inv_eps);
   __syncthreads();
 }
 

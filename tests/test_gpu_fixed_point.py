@@ -1,0 +1,78 @@
+"""The fixed-point form of the FP64 precision (fx64.cuh, lin_fx.cuh) against the FP64 kernels that LBO_OPT_KERNEL = 1 selects, at the
+sizes where it can go wrong: every N, a batch that spans several groups of
+the gain loop, few radial nodes, and inputs far from unit scale.
+
+Tolerance: both forms are within the stated bound of FP64, 4 u rms(r) max|L|
+(the ratio r = g/M over the grid), of the exact result, so they differ by at
+most twice that (64 stands for the rms of r = O(1) inputs, where other FP64
+roundings lead)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2503_09580_gb300 import lbo, workloads
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+U64 = 2.0 ** -53
+
+
+def apply(plan, params, g, quad=False):
+    tp, tg = torch.from_numpy(params).to(DEV), torch.from_numpy(g).to(DEV)
+    out = torch.full_like(tg, 7.0)
+    if quad:
+        plan.apply_quadratic(tg, out)
+    else:
+        plan.apply_linearized(tp, tg, out)
+    plan.sync()
+    return out.cpu().numpy()
+
+
+def ratio_rms(params, g, n, L, eps=1e-9):
+    a = workloads.velocity_axis(n, L)
+    r = np.zeros(params.shape[0])
+    for b, (rho, u1, u2, u3, th) in enumerate(params):
+        d2 = (a[:, None, None] - u1) ** 2 + (a[None, :, None] - u2) ** 2 + (a[None, None, :] - u3) ** 2
+        M = rho * (2 * np.pi * th) ** -1.5 * np.exp(-d2 / (2 * th))
+        keep = d2 / (2 * th) <= np.log(1 / eps) - 1.5 * np.log(2 * np.pi * th)
+        r[b] = np.sqrt(((g[b][keep] / M[keep]) ** 2).sum() / n ** 3)
+    return r
+
+
+@pytest.mark.parametrize("n,batch,J,noise", [(16, 1, 16, 0.0), (16, 130, 3, 1e-3), (24, 3, 24, 1e-3), (24, 1, 1, 0.0),
+                                             (32, 17, 32, 1e-3), (32, 1, 17, 0.0), (48, 2, 9, 1e-3), (64, 2, 5, 1e-3)])
+def test_linearized_matches_the_fp64_kernels(n, batch, J, noise):
+    L = 8.0
+    params, g = workloads.batched_instances(n, L, batch=batch, seed=70 + n, noise=noise)
+    a = apply(lbo.Plan(n, L, 0.74, J), params, g)
+    b = apply(lbo.Plan(n, L, 0.74, J, kernel=1), params, g)
+    tol = 2 * 4 * U64 * np.maximum(ratio_rms(params, g, n, L), 64.0)
+    for i in range(batch):
+        assert np.abs(a[i] - b[i]).max() <= tol[i] * np.abs(b[i]).max(), i
+
+
+def test_scale_and_degenerate_inputs():
+    """A power of two on g is exact; a zero field gives zero; a field or a
+    Maxwellian that is not finite gives NaN in its own instance alone; a
+    negative density and one far from 1 agree with the FP64 kernels."""
+    n, L = 16, 8.0
+    params, g = workloads.batched_instances(n, L, batch=6, seed=80, noise=1e-3)
+    plan, ref = lbo.Plan(n, L, 0.5, n), lbo.Plan(n, L, 0.5, n, kernel=1)
+    base = apply(plan, params, g)
+    for e in (200, -300):
+        assert np.array_equal(apply(plan, params, np.ldexp(g, e)), np.ldexp(base, e))
+    p2, g2 = params.copy(), g.copy()
+    g2[0] = 0.0
+    g2[1, 3, 4, 5] = np.nan
+    g2[2, 0, 0, 7] = np.inf
+    p2[3, 4] = -1.0
+    p2[4, 0] = -0.7
+    p2[5, 0] = 1e-100
+    a, b = apply(plan, p2, g2), apply(ref, p2, g2)
+    assert np.all(a[0] == 0)
+    for i in (1, 2, 3):
+        assert np.all(np.isnan(a[i])) and np.all(np.isnan(b[i]))
+    tol = 2 * 4 * U64 * np.maximum(ratio_rms(np.abs(p2), g2, n, L), 64.0)
+    for i in (4, 5):
+        assert np.abs(a[i] - b[i]).max() <= tol[i] * np.abs(b[i]).max()

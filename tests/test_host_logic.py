@@ -69,3 +69,22 @@ def test_register_fft32_against_a_direct_dft(tmp_path):
     assert res["double forward"] <= 8 * 2.0 ** -53 and res["double inverse"] <= 8 * 2.0 ** -53
     assert res["float forward"] <= 8 * 2.0 ** -24 and res["float inverse"] <= 8 * 2.0 ** -24
     assert res["twiddle"] <= 4 * 2.0 ** -53
+
+
+def test_fixed_point_arithmetic_against_long_double(tmp_path):
+    """The fixed-point products, pencil transforms and DCT-I (fx64.cuh) in units
+    of the last place.  A product leaves out yl tl (below 1/4) and takes two
+    floors balanced by 1: below 1.5; rounded once: below 1.  A transform's value
+    passes at most 5 products and its output sums 4 of them: rms below 1.5
+    sqrt(20); a DCT-I output sums at most H/2 doubled products.  The transforms
+    have no mean error beyond the 1/4 of a halving (N = 24), and keep zeros."""
+    out = subprocess.run([_build("fx64", tmp_path)], check=True, capture_output=True, text=True).stdout
+    res = {r[0]: (float(r[1]), float(r[2])) for r in (line.split() for line in out.strip().splitlines())}
+    assert res["mul"][0] < 1.5 and res["mul_signed"][0] < 1.5 and res["mul_signed_rounded"][0] < 1.0
+    assert abs(res["mul_signed_rounded"][1]) < 0.01
+    for n in (16, 24, 32):
+        for d in "fi":
+            err, bias = res["dft%d%s" % (n, d)]
+            assert err < 1.5 * 20 ** 0.5 and abs(bias) < (0.25 if n == 24 else 0.02), (n, d, err, bias)
+    for h in (8, 12, 16, 24, 32):
+        assert res["dct%d" % h][0] < 2 * 1.5 * h / 2, h
