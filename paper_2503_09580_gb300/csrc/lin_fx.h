@@ -25,8 +25,22 @@ struct Cache {
   const double* w;     // [B][N^3] InvFFT(FFT(M) omega)
 };
 
+// The hemisphere rule of Q(f,f) on the device, and optionally the loss
+// multiplier of Eq. (2.16) per half-spectrum position (FP64, positions of
+// fft.cuh) with a bound of its magnitude.
+struct QuadRule {
+  const double *gj, *sig, *wm;  // [J] radial nodes, [M][3] directions, [M] weights
+  int M;
+  double wmax;
+  const double* omega3;
+  double omega3_bound;
+};
+
 }  // namespace fx
 
+// Q(f,f) of FP64 on the integer pipe; ws: a buffer grown as needed
+lbo_status run_quadratic_fx(lbo_plan* p, const fx::QuadRule& rule, const double* f, double* out, int B, void** ws,
+                            size_t* ws_bytes);
 // L[g] of FP64 on the integer pipe (lin_fx_plan.cu)
 lbo_status run_linearized_fx(lbo_plan* p, const double* params, const double* g, double* out, int B, bool cached);
 lbo_status precompute_fx(lbo_plan* p, const double* params, int B);

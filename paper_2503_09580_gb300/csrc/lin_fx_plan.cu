@@ -1,5 +1,6 @@
 // Dispatch of the fixed-point form of the FP64 precision over N and over
-// groups of instances, and its tables (lin_fx.cuh has the kernels).
+// groups of instances, and its tables (lin_fx.cuh and quad_fx.cuh have the
+// kernels).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -15,6 +16,16 @@ namespace fx {
   lbo_status apply_##n(lbo_plan* p, const Tables& tb, const double* params, const double* g, double* out, int B,  \
                        int G, void* ws, const Cache* mc);                                                         \
   lbo_status precompute_##n(lbo_plan* p, const Tables& tb, const double* params, int B, void* ws, const Cache& mc);
+#define LBO_FX_QDECL(n)                                                                                            \
+  size_t q_workspace_bytes_##n(int B, int J, int M, bool position);                                               \
+  lbo_status q_apply_##n(lbo_plan* p, const Tables& tb, const QuadRule& rule, const double* f, double* out, int B, \
+                         void* ws);
+LBO_FX_QDECL(16)
+LBO_FX_QDECL(24)
+LBO_FX_QDECL(32)
+LBO_FX_QDECL(48)
+LBO_FX_QDECL(64)
+#undef LBO_FX_QDECL
 LBO_FX_DECL(16)
 LBO_FX_DECL(24)
 LBO_FX_DECL(32)
@@ -147,6 +158,28 @@ lbo_status ensure(void** ws, size_t* have, size_t bytes) {
   return LBO_OK;
 }
 
+size_t q_workspace_bytes(int N, int B, int J, int M, bool position) {
+  switch (N) {
+    case 16: return q_workspace_bytes_16(B, J, M, position);
+    case 24: return q_workspace_bytes_24(B, J, M, position);
+    case 32: return q_workspace_bytes_32(B, J, M, position);
+    case 48: return q_workspace_bytes_48(B, J, M, position);
+    default: return q_workspace_bytes_64(B, J, M, position);
+  }
+}
+
+lbo_status q_apply_part(lbo_plan* p, const Tables& tb, const QuadRule& rule, const double* f, double* out, int B,
+                        void* ws) {
+  switch (p->N) {
+    case 16: return q_apply_16(p, tb, rule, f, out, B, ws);
+    case 24: return q_apply_24(p, tb, rule, f, out, B, ws);
+    case 32: return q_apply_32(p, tb, rule, f, out, B, ws);
+    case 48: return q_apply_48(p, tb, rule, f, out, B, ws);
+    case 64: return q_apply_64(p, tb, rule, f, out, B, ws);
+    default: return LBO_EUNSUPPORTED;
+  }
+}
+
 }  // namespace
 }  // namespace fx
 
@@ -187,6 +220,22 @@ lbo_status precompute_fx(lbo_plan* p, const double* params, int B) {
   p->last_launches = 0;
   for (int b0 = 0; b0 < B && st == LBO_OK; b0 += part)
     st = fx::precompute_part(p, tb, params + 5 * (size_t)b0, std::min(part, B - b0), fx::cache_at(p, B, b0));
+  return st;
+}
+
+lbo_status run_quadratic_fx(lbo_plan* p, const fx::QuadRule& rule, const double* f, double* out, int B, void** ws,
+                            size_t* ws_bytes) {
+  fx::Tables tb;
+  lbo_status st = fx::tables(p, &tb);
+  const int part = fx::part_size(p, B);
+  if (st == LBO_OK)
+    st = fx::ensure(ws, ws_bytes, fx::q_workspace_bytes(p->N, part, p->J, rule.M, rule.omega3 != nullptr));
+  const size_t n3 = (size_t)p->N * p->N * p->N;
+  p->last_launches = 0;
+  for (int b0 = 0; b0 < B && st == LBO_OK; b0 += part)
+    st = fx::q_apply_part(p, tb, rule, f + b0 * n3, out + b0 * n3, std::min(part, B - b0), *ws);
+  if (st == LBO_OK && (p->mass_fix || p->moment_fix))
+    st = launch_fixes(p, out, B, p->N, 2.0 * p->L / p->N, p->stream, &p->last_launches);
   return st;
 }
 

@@ -1,0 +1,152 @@
+// build-variants: LBO_FX_N=16 LBO_FX_N=24 LBO_FX_N=32 LBO_FX_N=48 LBO_FX_N=64
+//
+// Q(f,f) in the FP64 precision in 64-bit fixed point on the integer pipe
+// (quad_fx.cuh), one translation unit per N; lin_fx_plan.cu dispatches to the
+// functions defined here.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "lin_fx.h"
+#include "quad_fx.cuh"
+
+#define LBO_CAT_(a, b) a##b
+#define LBO_CAT(a, b) LBO_CAT_(a, b)
+
+namespace lbo {
+namespace fx {
+
+namespace {
+
+constexpr int N = LBO_FX_N;
+constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, T = Geo<N>::T;
+constexpr size_t H = (size_t)N * NC, n3 = (size_t)N * N * N;
+constexpr int ACC_WARPS = 8, PPC = PlanesPPC<N>::v, CPPC = CombinePPC<N>::v;
+
+// How a call is cut: G instances at a time whose J plane spectra PW stay below
+// 512 MB; of their (instance, node) pairs as many per launch, and of a pair's M
+// hemisphere nodes as many, as 1 GB of Z holds.
+struct Cut {
+  int G, mc, pairs;
+  Cut(int B, int J, int M) {
+    const size_t z = sizeof(ci64) * n3;
+    G = (int)std::min<size_t>(B, std::max<size_t>(1, ((size_t)512 << 20) / (sizeof(ci64) * H * J)));
+    mc = (int)std::min<size_t>(M, std::max<size_t>(1, ((size_t)1 << 30) / z));
+    pairs = (int)std::min<size_t>((size_t)G * J, std::max<size_t>(1, ((size_t)1 << 30) / (z * mc)));
+  }
+};
+
+struct Buffers {
+  ci64 *R, *F, *PW, *Z, *tab;
+  i64 *accG, *om3;
+  double *BPh, *BP;
+  float* rm;
+  int *eR, *EF, *EPh, *EC, *bad, *EP, *accE;
+  size_t bytes;
+  Buffers(void* base, size_t B, size_t J, size_t M, const Cut& c, bool position) {
+    unsigned char* p = (unsigned char*)base;
+    auto take = [&](auto*& ptr, size_t count) {
+      ptr = (std::remove_reference_t<decltype(ptr)>)p;
+      p += (count * sizeof(*ptr) + 255) / 256 * 256;
+    };
+    const bool rest = (size_t)c.mc < M;
+    take(R, B * H);
+    take(F, 2 * B * H);
+    take(PW, c.G * J * H);
+    take(Z, (size_t)c.pairs * c.mc * n3);
+    take(tab, J * M * 3 * N);
+    take(accG, rest ? c.pairs * n3 : 0);
+    take(om3, position ? H : 0);
+    take(BPh, B * N);
+    take(BP, c.G * J * N);
+    take(rm, B * HC * NC);
+    take(eR, B * NC);
+    take(EF, B);
+    take(EPh, B * N);
+    take(EC, 2 * B * NC);
+    take(bad, B);
+    take(EP, c.G * J * N);
+    take(accE, rest ? (size_t)c.pairs * N : 0);
+    bytes = (size_t)(p - (unsigned char*)base);
+  }
+};
+
+template <typename K>
+void smem_of(K kernel, size_t bytes) { raise_smem_limit((const void*)kernel, bytes); }
+
+}  // namespace
+
+size_t LBO_CAT(q_workspace_bytes_, LBO_FX_N)(int B, int J, int M, bool position) {
+  return Buffers(nullptr, B, J, M, Cut(B, J, M), position).bytes;
+}
+
+lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const QuadRule& rule, const double* f, double* out,
+                                       int B, void* ws) {
+  cudaStream_t s = p->stream;
+  const int J = p->J, M = rule.M;
+  const Cut cut(B, J, M);
+  const Buffers w(ws, B, J, M, cut, rule.omega3 != nullptr);
+  cudaError_t e = cudaMemsetAsync(w.bad, 0, sizeof(int) * B, s);
+  if (e != cudaSuccess) return cuda_fail(e, "fixed-point flags");
+  const double pi = 3.141592653589793238462643383279502884;
+  // phi_j carries 4 pi^2 w_j B_j s_j / N^6 (one 1 / N^3 for T+ or T-, one for
+  // the last transform); Eq. (2.14): 16 pi^2, and T+ T- a second 1 / N^3
+  const double c0 = 4.0 / ((double)N * N * N);
+  int ke = 0;
+  const double top = std::frexp(std::sqrt(rule.wmax * c0), &ke);  // top 2^ke, top in [0.5, 1)
+  (void)top;
+  const double c = std::scalbn(c0, -2 * ke);
+  LBO_LAUNCH(p, "q_fx_phase_table", s, k_q_phase_table<N>, J * M, 3 * N, 0, rule.gj, rule.sig, rule.wm, M, pi, 2.0 * p->L,
+             c, w.tab);
+  int launches = 5;
+  const i64* omega = tb.omega;
+  int omega_exp = tb.omega_exp;
+  if (rule.omega3) {
+    omega = w.om3;
+    omega_exp = 61 - std::ilogb(rule.omega3_bound);
+    LBO_LAUNCH(p, "q_fx_multipliers", s, k_q_position_multipliers<N>, 152, 256, 0, rule.omega3, omega_exp, w.om3);
+    launches += 1;
+  }
+  // F = FFT(f); InvFFT_1(F omega)
+  smem_of(k_fwd_planes<N, PPC>, Planes<N, PPC>::BYTES);
+  LBO_LAUNCH(p, "q_fx_plane_fwd", s, (k_fwd_planes<N, PPC>), dim3(N / PPC, B, 1), (Planes<N, PPC>::THREADS),
+             (Planes<N, PPC>::BYTES), f, (const double*)nullptr, 0, 0, w.F, w.EPh, w.BPh, w.bad);
+  LBO_LAUNCH(p, "q_fx_axis1_head", s, k_axis1_head<N>, dim3((NC * T + 63) / 64, B, 2), 64, 0, w.F, w.EPh,
+             (const ci64*)nullptr, (const int*)nullptr, omega, rule.omega3 ? 1 : 0, omega_exp, 0, w.R, w.eR, w.rm, w.EC, 0);
+  LBO_LAUNCH(p, "q_fx_rescale", s, k_q_rescale<N>, dim3((NC + 63) / 64, B), 64, 0, w.R, w.eR, w.rm, w.EF);
+  smem_of(k_q_plane<N>, GeoQ<N>::BYTES);
+  smem_of(k_axis1_acc<N, ACC_WARPS>, acc_smem<N, ACC_WARPS>(256));
+  // head room of the sum over m: products below 2^60
+  int guard = 0;
+  while ((2 << guard) < M) ++guard;
+  for (int b0 = 0; b0 < B; b0 += cut.G) {
+    const int n = std::min(cut.G, B - b0);
+    const ci64* R = w.R + b0 * H;
+    for (int q0 = 0; q0 < n * J; q0 += cut.pairs) {
+      const int np = std::min(cut.pairs, n * J - q0);
+      for (int m0 = 0; m0 < M; m0 += cut.mc) {
+        const int mc = std::min(cut.mc, M - m0);
+        LBO_LAUNCH(p, "q_fx_axis1_phase", s, k_q_axis1<N>, dim3((NC * T + 31) / 32, mc, np), 32, 0, R, w.tab, J, M, m0, q0,
+                   w.Z);
+        LBO_LAUNCH(p, "q_fx_plane_prod", s, k_q_plane<N>, dim3(N / GeoQ<N>::PPC, np), GeoQ<N>::THREADS, GeoQ<N>::BYTES,
+                   w.Z, w.EF + b0, J, mc, q0, m0 == 0 ? 1 : 0, m0 + mc == M ? 1 : 0, guard, ke, w.accG, w.accE, w.PW, w.EP,
+                   w.BP);
+        launches += 2;
+      }
+    }
+    LBO_LAUNCH(p, "q_fx_axis1_fwd_acc", s, (k_axis1_acc<N, ACC_WARPS>), dim3((NC * T + 31) / 32, n), 32 * ACC_WARPS,
+               (acc_smem<N, ACC_WARPS>(J)), w.PW, w.EP, w.BP, tb.phi, tb.phi_exp, tb.phi_max, w.F + b0 * H,
+               w.EC + b0 * (size_t)NC, J);
+    launches += 1;
+  }
+  using C = Combine<N, CPPC, QUAD>;
+  smem_of(k_combine_planes<N, CPPC, QUAD>, C::BYTES);
+  LBO_LAUNCH(p, "q_fx_combine", s, (k_combine_planes<N, CPPC, QUAD>), dim3(N / CPPC, B), C::THREADS, C::BYTES,
+             (const double*)nullptr, f, w.F, w.EC, (const double*)nullptr, w.bad, out);
+  p->last_launches += launches;
+  e = cudaGetLastError();
+  return e == cudaSuccess ? LBO_OK : cuda_fail(e, "fixed-point quadratic launch");
+}
+
+}  // namespace fx
+}  // namespace lbo

@@ -15,6 +15,7 @@
 #include <cmath>
 #include <vector>
 
+#include "lin_fx.h"
 #include "quad_generic.cuh"
 
 namespace lbo {
@@ -178,13 +179,15 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
   const size_t N = p->N, H = N * N * (N / 2 + 1), n3 = N * N * N;
   const int M = (int)qs->wm.size();
   const size_t rb = generic_real_bytes(p->precision);
-  const size_t MB = fused ? 0 : (size_t)q_chunk(B, M, (int)N, rb);
+  // FP64 in fixed point on the integer pipe (quad_fx.cuh), its own buffers
+  const bool fixed = p->precision == LBO_PREC_FP64 && p->kernel_choice == 0;
+  const size_t MB = fused || fixed ? 0 : (size_t)q_chunk(B, M, (int)N, rb);
   // FP64 at N = 32 (register kernels): the phase-factor table after the chunk buffers
   const size_t ptab = p->precision == LBO_PREC_FP64 && N == 32 && p->kernel_choice != 2
                           ? (size_t)p->J * M * 3 * N * 2 * sizeof(double) : 0;
   const size_t need = fused ? quad_fused32_workspace_bytes(B, G)
                             : (size_t)B * (4 * H * 2 * rb + 3 * n3 * rb) + MB * (size_t)B * (2 * H * 2 * rb + n3 * rb) + ptab;
-  if (need > qs->ws_bytes) {
+  if (!fixed && need > qs->ws_bytes) {
     if (qs->ws) cudaFree(qs->ws);
     qs->ws = nullptr;
     qs->ws_bytes = 0;
@@ -224,6 +227,15 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
     lbo_status st = ensure_omega_quadrature(p, qs);
     if (st != LBO_OK) return st;
     omq = qs->d_omq;
+  }
+  if (fixed) {
+    const double* dsig = qs->d_gsw + p->J;
+    double bound = 0.0;
+    for (int j = 0; j < p->J; ++j) bound += std::fabs(p->wj[j] * p->Bj[j]);
+    bound *= 16.0 * 3.141592653589793 * 3.141592653589793 / ((double)p->N * p->N * p->N);
+    const fx::QuadRule rule{qs->d_gsw, dsig, dsig + 3 * M, M, *std::max_element(qs->wm.begin(), qs->wm.end()),
+                            (const double*)omq, bound};
+    return run_quadratic_fx(p, rule, f, out, B, &qs->ws, &qs->ws_bytes);
   }
   switch (p->precision) {
     case LBO_PREC_FP64: return dispatch_q<double>(p, qs, f, out, B, p->d_phi64, p->d_omega64, omq);

@@ -1,11 +1,14 @@
-"""The fixed-point form of the FP64 precision (fx64.cuh, lin_fx.cuh) against the FP64 kernels that LBO_OPT_KERNEL = 1 selects, at the
+"""The fixed-point form of the FP64 precision (fx64.cuh, lin_fx.cuh,
+quad_fx.cuh) against the FP64 kernels that LBO_OPT_KERNEL = 1 selects, at the
 sizes where it can go wrong: every N, a batch that spans several groups of
 the gain loop, few radial nodes, and inputs far from unit scale.
 
 Tolerance: both forms are within the stated bound of FP64, 4 u rms(r) max|L|
 (the ratio r = g/M over the grid), of the exact result, so they differ by at
 most twice that (64 stands for the rms of r = O(1) inputs, where other FP64
-roundings lead)."""
+roundings lead); Q transforms f itself, whose two forms are each within
+2^-53 times the 3 log2 N^3 additions a value passes, times the 8 sqrt(J M)
+of random sums over nodes."""
 import numpy as np
 import pytest
 
@@ -76,3 +79,24 @@ def test_scale_and_degenerate_inputs():
     tol = 2 * 4 * U64 * np.maximum(ratio_rms(np.abs(p2), g2, n, L), 64.0)
     for i in (4, 5):
         assert np.abs(a[i] - b[i]).max() <= tol[i] * np.abs(b[i]).max()
+
+
+@pytest.mark.parametrize("n,batch,J,p,kw", [(16, 5, 16, 1, {}), (16, 1, 3, 5, {"q_sinc_quadrature": 1}), (24, 3, 24, 2, {}),
+                                            (32, 3, 32, 4, {}), (32, 2, 5, 2, {"q_sinc_quadrature": 1}), (48, 2, 4, 3, {}),
+                                            (64, 1, 12, 4, {})])
+def test_quadratic_matches_the_fp64_kernels(n, batch, J, p, kw):
+    L = 8.0
+    _, g = workloads.batched_instances(n, L, batch=batch, seed=90 + n, noise=0.0)
+    params = np.zeros((batch, 5))
+    a = apply(lbo.Plan(n, L, 0.5, J, hemisphere_p=p, **kw), params, g, quad=True)
+    b = apply(lbo.Plan(n, L, 0.5, J, hemisphere_p=p, kernel=1, **kw), params, g, quad=True)
+    tol = 2 * U64 * 3 * 3 * np.log2(n) * 8
+    for i in range(batch):
+        assert np.abs(a[i] - b[i]).max() <= tol * np.abs(b[i]).max(), i
+    g[0] = 0.0
+    g[-1, 1, 2, 3] = np.nan
+    c = apply(lbo.Plan(n, L, 0.5, J, hemisphere_p=p, **kw), params, g, quad=True)
+    assert np.all(np.isnan(c[-1]))
+    if batch > 1:
+        assert np.all(c[0] == 0)
+        assert all(np.array_equal(c[i], a[i]) for i in range(1, batch - 1))
