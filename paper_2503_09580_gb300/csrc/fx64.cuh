@@ -92,7 +92,17 @@ FX_FN i64 mul_signed(i64 y, Mult t, int neg) {
   const int c = (int)(umulhi32(yl, (unsigned)t.th) - (yl & (unsigned)neg)) + mulhi32(yh, t.tl) + 1;
   return (i64)yh * t.th + (i64)c;
 }
-// The same rounded once, from the exact sum of the cross products: unbiased
+// y m 2^(b - 64) for a multiplier 0 <= m < 2^60 split at bit 31 (pack_finer), 1 <= b
+// <= 31: b more bits than mul() keeps, all four partial products taken.
+FX_FN i64 pack_finer(i64 m) { return (i64)(((u64)m >> 31) << 32 | ((u64)m & 0x7fffffffULL)); }
+FX_FN i64 mul_finer(i64 y, i64 packed, int b) {
+  const unsigned yl = (unsigned)(u64)y, th = (unsigned)((u64)packed >> 32), tl = (unsigned)(u64)packed;
+  const int yh = (int)(y >> 32);
+  const u64 t0 = (u64)(yl >> 1) * th + umulhi32(yl, tl);
+  const i64 t1 = (i64)yh * (int)tl + (i64)t0;
+  return (i64)((u64)((i64)yh * (int)th) << (b - 1)) + ((t1 + ((i64)1 << (31 - b))) >> (32 - b));
+}
+// mul_signed() rounded once, from the exact sum of the cross products: unbiased
 // also where th = 0 (a multiplier far below its table's largest entry), where
 // the + 1 of mul_signed() would add half a unit to every product.
 FX_FN i64 mul_signed_rounded(i64 y, Mult t, int neg) {

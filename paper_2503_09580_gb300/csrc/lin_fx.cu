@@ -31,7 +31,7 @@ struct Buffers {
   i64* mh;
   double *inst, *BPh;
   float* rm;
-  int *eR, *me, *eM, *EPh, *EC, *bad;
+  int *eR, *em, *eM, *EPh, *EC, *bad;
   // of G instances
   ci64* W;
   i64* U;
@@ -52,7 +52,7 @@ struct Buffers {
     take(BPh, 2 * B * N);
     take(rm, B * HC * NC);
     take(eR, B * NC);
-    take(me, B * 3 * N);
+    take(em, B * N);
     take(eM, B * 3);
     take(EPh, 2 * B * N);
     take(EC, 3 * B * NC);
@@ -74,8 +74,8 @@ template <typename K>
 void smem_of(K kernel, size_t bytes) { raise_smem_limit((const void*)kernel, bytes); }
 
 void launch_instance(lbo_plan* p, const Buffers& w, const double* params, int* bad, int B, const char* name) {
-  LBO_LAUNCH(p, name, p->stream, k_instance<N>, B, kInstanceThreads<N>, 0, params, 2.0 * p->L / N, std::log(1.0 / p->eps), w.inst, w.me,
-             w.MH, w.eM, bad);
+  LBO_LAUNCH(p, name, p->stream, k_instance<N>, B, kInstanceThreads<N>, 0, params, 2.0 * p->L / N, std::log(1.0 / p->eps), w.inst, w.em,
+             bad);
 }
 
 void launch_uhat(lbo_plan* p, const double* inst, i64* U, int* eU, int* bad, int B, const char* name) {
@@ -103,7 +103,7 @@ template <int P>
 void launch_planes(lbo_plan* p, const Buffers& w, int b0, int B) {
   smem_of(k_plane<N, P>, Planes<N, P>::BYTES);
   LBO_LAUNCH(p, "fx_plane_inv_mh_fwd", p->stream, (k_plane<N, P>), dim3(N / P, p->J, B), (Planes<N, P>::THREADS),
-             (Planes<N, P>::BYTES), w.W, w.EA, w.mh + b0 * n3, w.me + b0 * 3 * N, w.EP, w.BP);
+             (Planes<N, P>::BYTES), w.W, w.EA, w.mh + b0 * n3, w.em + b0 * N, w.EP, w.BP);
 }
 
 void launch_head(lbo_plan* p, const Tables& tb, const Buffers& w, int B, int z0, int count, const char* name) {
@@ -138,7 +138,7 @@ lbo_status LBO_CAT(apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const double
                      : cudaMemsetAsync(w.bad, 0, sb, s);
   if (e != cudaSuccess) return cuda_fail(e, "fixed-point flags");
   launch_instance(p, w, params, w.bad, B, "fx_instance");
-  LBO_LAUNCH(p, "fx_mh_table", s, k_mh<N>, dim3(N, B), 256, 0, w.inst, w.mh);
+  LBO_LAUNCH(p, "fx_mh_table", s, k_mh<N>, dim3(N + 1, B), 256, 0, w.inst, w.em, w.mh, w.MH, w.eM);
   // r^ = FFT(r); InvFFT_1 of g^ omega and of M^ omega
   smem_of(k_fwd_planes<N, PPC>, Planes<N, PPC>::BYTES);
   LBO_LAUNCH(p, "fx_plane_fwd", s, (k_fwd_planes<N, PPC>), dim3(N / PPC, B, 2), (Planes<N, PPC>::THREADS),
@@ -180,10 +180,11 @@ lbo_status LBO_CAT(precompute_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const d
                                           const Cache& mc) {
   const Buffers w(ws, B, 0, p->J, false);
   launch_instance(p, w, params, (int*)mc.bad, B, "cache_fx_instance");
+  LBO_LAUNCH(p, "cache_fx_mh_table", p->stream, k_mh<N>, dim3(N + 1, B), 256, 0, w.inst, w.em, w.mh, w.MH, w.eM);
   launch_uhat(p, w.inst, (i64*)mc.U, (int*)mc.eU, (int*)mc.bad, B, "cache_fx_uhat");
   launch_head(p, tb, w, B, 2, 1, "cache_fx_axis1_head");
   launch_combine<FACTOR>(p, w, nullptr, nullptr, mc.bad, (double*)mc.w, B, "cache_fx_combine");
-  p->last_launches += 4;
+  p->last_launches += 5;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LBO_OK : cuda_fail(e, "fixed-point cache launch");
 }

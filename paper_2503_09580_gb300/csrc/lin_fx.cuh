@@ -8,7 +8,7 @@
 // nodes, and a group is chosen so that its half spectra stay in the L2 cache:
 //
 //   k_instance       per-instance tables (all exponentials)
-//   k_mh             the table of M^h
+//   k_mh             the table of M^h, the 1-D transforms of M's factors
 //   k_fwd_planes     axes 3 and 2 of FFT(r) and FFT(g)
 //   k_axis1_head     axis 1 of r^; InvFFT_1(FFT(g) omega), InvFFT_1(FFT(M) omega)
 //   k_uhat           u^_j of a unit on its (N/2+1)^3 octant (three DCT-I passes)
@@ -31,12 +31,15 @@ namespace fx {
 template <int N>
 struct Geo {
   static constexpr int HC = N / 2 + 1, NC = N * HC;
-  static constexpr int T = N > 32 ? 2 : 1;  // threads per pencil
+  static constexpr int T = N >= 32 ? 2 : 1;  // threads per pencil
   static constexpr int V = N / T;           // values per thread
+  // row stride of a plane in shared memory: odd, or 2 mod 8 for pairs of
+  // threads, so that the row pass is free of bank conflicts
+  static constexpr int RS = T == 2 ? HC + 1 : HC;
   static constexpr int PEN = N / 2;         // pencils per plane and pass
   static constexpr int TPP = PEN * T;       // threads per plane
   // the threads of a plane are consecutive lanes of one warp
-  static constexpr bool WARP = TPP == 8 || TPP == 16;
+  static constexpr bool WARP = TPP == 8 || TPP == 16 || TPP == 32;
 };
 
 constexpr int kSumBits = 60;       // sum(|re| + |im|) of a pencil before its transform, at most 2^60
@@ -148,6 +151,24 @@ __device__ __forceinline__ void shift_all(ci64 (&x)[V], int s) {
     for (int i = 0; i < V; ++i) x[i] = ci64{(i64)((u64)x[i].x << -s), (i64)((u64)x[i].y << -s)};
   }
 }
+// The same floored: where the following inverse transforms gather the mean
+// error in the corner of the grid and M^h takes it away.
+template <int V>
+__device__ __forceinline__ void shift_floor(ci64 (&x)[V], int s) {
+  if (s > 0) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) x[i] = ci64{x[i].x >> s, x[i].y >> s};
+  } else if (s < 0) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) x[i] = ci64{(i64)((u64)x[i].x << -s), (i64)((u64)x[i].y << -s)};
+  }
+}
+// round(x 2^-s), 0 <= s <= 63 (the PTX shift by 0xffffffff gives 0)
+__device__ __forceinline__ i64 shift_right(i64 x, int s) {
+  i64 half;
+  asm("shl.b64 %0, %1, %2;" : "=l"(half) : "l"(1LL), "r"(s - 1));
+  return (x + half) >> s;
+}
 // 2^-e as a float, 0 beyond its normal range (e >= 0)
 __device__ __forceinline__ float exp2_neg(int e) { return e > 126 ? 0.f : __uint_as_float((unsigned)(127 - e) << 23); }
 // x 2^e as FP64, rounded to nearest even; the integer pipe does it (a
@@ -184,15 +205,13 @@ struct Inst {
   static constexpr int EM = 0;           // [3][N] factors of M (fill_maxwellian_tables)
   static constexpr int EI = 3 * N;       // [3][N] factors of 1/M (fill_ratio_tables)
   static constexpr int SQ = 6 * N;       // [3][N] (v_i - u_d)^2, every operation rounded
-  static constexpr int EH = 9 * N;       // [3][N] mantissas of the factors of |M^h|, in [1, 2) or 0
+  static constexpr int EH = 9 * N;       // [3][N] factors of |M^h|
   static constexpr int MG = 12 * N;      // [N/2+1] exp(-(i h)^2 / theta), then |rho| (pi theta)^(-3/2)
   static constexpr int DSTAR = 12 * N + N / 2 + 2;  // the cut-off's distance (fill_ratio_tables)
   static constexpr int SIZE = DSTAR + 1;
 };
-constexpr int kZeroShift = 4096;  // exponent distance of a factor that underflowed to 0
 
-// inst as above; me[b][d][i]: the exponents of M^h's factors (see k_mh); MH[b][d]
-// [k] 2^eM[b][d] = the 1-D transforms of M's factors, whose product is FFT(M).
+// inst as above; em[b][i1]: exponent of the plane i1 of M^h (see k_mh).
 // |rho| in M^h and in the weights of u^_j: multipliers are not negative, and
 // L^+ has the product of the two.
 // bad[b]: 1 where a factor is not finite (the output is then NaN).
@@ -201,23 +220,19 @@ template <int N>
 constexpr int kInstanceThreads = (9 * N + N / 2 + 1 + 3 + 31) / 32 * 32;
 template <int N>
 __global__ void __launch_bounds__(kInstanceThreads<N>) k_instance(const double* __restrict__ params, double h, double log_inv_eps,
-                                                  double* __restrict__ inst, int* __restrict__ me,
-                                                  ci64* __restrict__ MH, int* __restrict__ eM, int* __restrict__ bad) {
-  constexpr int T = Geo<N>::T, V = Geo<N>::V, HC = Geo<N>::HC;
+                                                  double* __restrict__ inst, int* __restrict__ em1,
+                                                  int* __restrict__ bad) {
+  constexpr int HC = Geo<N>::HC;
   // tasks: every exponential, power and the cut-off's distance in a thread of
   // its own, side by side, then the products
   constexpr int TI = 3 * N, TH = 6 * N, TG = 9 * N, TP = 9 * N + HC;  // ends of M, 1/M, M^h, M^g
   static_assert(TP + 3 <= kInstanceThreads<N>, "one thread per task");
-  __shared__ double em[3 * N], pre[2];
-  __shared__ int top[3];
-  __shared__ unsigned topm[3];
+  __shared__ double pre[2];
+  __shared__ unsigned long long top[3];  // largest factor of M^h per axis (bits of a positive double)
   const int b = blockIdx.x, t = threadIdx.x;
   const InstanceParams q = load_params(params, b);
   double* I = inst + (size_t)b * Inst<N>::SIZE;
-  if (t < 3) {
-    top[t] = kZeroExp;
-    topm[t] = 0;
-  }
+  if (t < 3) top[t] = 0;
   double e = 0.0;
   const int ti = t % (3 * N), d = ti / N;  // axis and index of the factor tasks
   if (t < TG) {
@@ -245,13 +260,10 @@ __global__ void __launch_bounds__(kInstanceThreads<N>) k_instance(const double* 
     I[Inst<N>::DSTAR] = cut_distance(q.theta, log_inv_eps);
   }
   __syncthreads();
-  int ex = kZeroExp;
   if (t < TI) {
     if (d == 0) e *= pre[0];
-    em[ti] = e;
     I[Inst<N>::EM + ti] = e;
     if (!isfinite(e)) atomicOr(bad + b, 1);
-    atomicMax(&topm[d], (unsigned)__double2hiint(e) & 0x7fffffffu);
   } else if (t < TH) {
     if (d == 0) e /= pre[0];
     I[Inst<N>::EI + ti] = e;
@@ -259,46 +271,55 @@ __global__ void __launch_bounds__(kInstanceThreads<N>) k_instance(const double* 
     if (d == 0) e *= pre[1];
     e = fabs(e);
     if (!isfinite(e)) atomicOr(bad + b, 1);
-    if (isfinite(e) && e != 0.0) ex = ilogb(e);
-    atomicMax(&top[d], ex);
-    I[Inst<N>::EH + ti] = ex == kZeroExp ? 0.0 : scalbn(e, -ex);
+    else atomicMax(&top[d], (unsigned long long)__double_as_longlong(e));
+    I[Inst<N>::EH + ti] = isfinite(e) ? e : 0.0;
   }
   __syncthreads();
-  if (t >= TH && t < TG)
-    me[b * 3 * N + ti] = d == 0 ? ex + top[1] + top[2] - 59 : (ex == kZeroExp ? kZeroShift : top[d] - ex);
-  if (t >= 32) return;
-  const int h2 = T == 2 ? t & 1 : 0, dm = min(t / T, 2);
-  const bool fin = topm[dm] < 0x7ff00000u;
-  const int E = (int)(topm[dm] >> 20) - 1023 - 57;  // the largest factor in [2^57, 2^58)
-  ci64 x[V];
-#pragma unroll
-  for (int i = 0; i < V; ++i) x[i] = ci64{fin ? to_fixed(em[dm * N + idx_parity<N>(i, h2)], E) : 0, 0};
-  const int s = shift_for(pencil_sum<N>(abs_sum<V>(x)), kSumBits);
-  shift_all<V>(x, s);
-  dft_time<N, false>(x, h2);
-  if (t < 3 * T) {
-#pragma unroll
-    for (int i = 0; i < V; ++i) MH[((size_t)b * 3 + dm) * N + idx_halves<N>(i, h2)] = x[i];
-    if (h2 == 0) eM[b * 3 + dm] = E + s;
+  if (t >= TH && t < TH + N) {
+    const double m = (e * __longlong_as_double((i64)top[1])) * __longlong_as_double((i64)top[2]);
+    em1[b * N + ti] = m > 0.0 && isfinite(m) ? ilogb(m) - 59 : 0;
   }
 }
 
-// |M^h(v)| = mh[b][i1][i3][i2] 2^(me[b][0][i1] - me[b][1][i2] - me[b][2][i3]): the
-// product of the mantissas of the three separable factors, in [2^59, 2^62), as
-// a multiplier (pack_mult), and the factors' exponents (axes 2 and 3 below
-// their largest, so >= 0).  The product psi_j M^h is so rounded relative to
-// each value of M^h: psi_j is largest in the tails, where M^h is smallest, and
-// one unit of the largest product there would drown the others.  i2 runs
-// fastest so that the row threads of k_plane read consecutive entries.
-// grid = (N, B), block = 256.
+// |M^h(v)| = mh[b][i1][i3][i2] 2^em[b][i1] as a multiplier (pack_finer), every
+// plane's largest entry in [2^59, 2^60).  i2 runs fastest so that the row
+// threads of k_plane read consecutive entries.  The last block of an instance:
+// MH[b][d][k] 2^eM[b][d] = the 1-D transforms of M's factors, whose product is
+// FFT(M).
+// grid = (N + 1, B), block = 256.
 template <int N>
-__global__ void __launch_bounds__(256) k_mh(const double* __restrict__ inst, i64* __restrict__ mh) {
-  const int b = blockIdx.y, i1 = blockIdx.x;
-  const double* eh = inst + (size_t)b * Inst<N>::SIZE + Inst<N>::EH;
-  i64* dst = mh + ((size_t)b * N + i1) * N * N;
-  const double e1 = eh[i1] * 0x1p59;
-  for (int t = threadIdx.x; t < N * N; t += blockDim.x)
-    dst[t] = pack_mult(__double2ll_rn((e1 * eh[N + t % N]) * eh[2 * N + t / N]));
+__global__ void __launch_bounds__(256) k_mh(const double* __restrict__ inst, const int* __restrict__ em,
+                                            i64* __restrict__ mh, ci64* __restrict__ MH, int* __restrict__ eM) {
+  const int b = blockIdx.y, i1 = blockIdx.x, t = threadIdx.x;
+  const double* I = inst + (size_t)b * Inst<N>::SIZE;
+  if (i1 < N) {
+    const double* eh = I + Inst<N>::EH;
+    const int E = em[b * N + i1];
+    i64* dst = mh + ((size_t)b * N + i1) * N * N;
+    for (int e = t; e < N * N; e += 256)
+      dst[e] = pack_finer(to_fixed((eh[i1] * eh[N + e % N]) * eh[2 * N + e / N], E));
+    return;
+  }
+  constexpr int T = Geo<N>::T, V = Geo<N>::V;
+  if (t >= 32) return;
+  const int h = T == 2 ? t & 1 : 0, d = min(t / T, 2);
+  const double* m = I + Inst<N>::EM + d * N;
+  unsigned top = 0;
+#pragma unroll 8
+  for (int i = 0; i < N; ++i) top = max(top, (unsigned)__double2hiint(m[i]) & 0x7fffffffu);
+  const bool fin = top < 0x7ff00000u;
+  const int E = (int)(top >> 20) - 1023 - 57;  // the largest factor in [2^57, 2^58)
+  ci64 x[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) x[i] = ci64{fin ? to_fixed(m[idx_parity<N>(i, h)], E) : 0, 0};
+  const int s = shift_for(pencil_sum<N>(abs_sum<V>(x)), kSumBits);
+  shift_all<V>(x, s);
+  dft_time<N, false>(x, h);
+  if (t < 3 * T) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) MH[((size_t)b * 3 + d) * N + idx_halves<N>(i, h)] = x[i];
+    if (h == 0) eM[b * 3 + d] = E + s;
+  }
 }
 
 // ------------------------------------------------------------ u^_j
@@ -559,7 +580,9 @@ struct CombinePPC { static constexpr int v = N == 32 ? 2 : (N < 32 ? 4 : 1); };
 template <int N, int PPC>
 struct Planes {
   static constexpr int THREADS = Geo<N>::TPP * PPC;
-  static constexpr size_t BYTES = sizeof(ci64) * (size_t)PPC * N * Geo<N>::HC;
+  // blocks per SM asked of the compiler: 168 registers where a thread holds 16 values
+  static constexpr int BLOCKS = Geo<N>::V == 16 ? 384 / THREADS : 1;
+  static constexpr size_t BYTES = sizeof(ci64) * (size_t)PPC * N * Geo<N>::RS;
 };
 
 // Barrier and maximum over the threads of a plane.  Where a plane is part of
@@ -599,10 +622,11 @@ __device__ __forceinline__ PlaneThread plane_thread(int t) {
 
 // shift by the plane's largest pencil sum (returned); E is the values' exponent
 template <int N>
-__device__ __forceinline__ float normalise(ci64 (&x)[Geo<N>::V], int& s, int& E, unsigned* slot) {
+__device__ __forceinline__ float normalise(ci64 (&x)[Geo<N>::V], int& s, int& E, unsigned* slot, bool round) {
   const float top = plane_max<N>(pencil_sum<N>(abs_sum<Geo<N>::V>(x)), slot);
   s = shift_for(top, kSumBits);
-  shift_all<Geo<N>::V>(x, s);
+  if (round) shift_all<Geo<N>::V>(x, s);
+  else shift_floor<Geo<N>::V>(x, s);
   E += s;
   return top;
 }
@@ -630,16 +654,16 @@ __device__ __forceinline__ void pencil_inverse(ci64 (&x)[Geo<N>::V], int h, bool
 template <int N>
 __device__ __forceinline__ void store_columns(const ci64 (&x)[Geo<N>::V], const PlaneThread& t, ci64* Bs) {
 #pragma unroll
-  for (int i = 0; i < Geo<N>::V; ++i) Bs[idx_halves<N>(i, t.h) * Geo<N>::HC + t.q] = x[i];
+  for (int i = 0; i < Geo<N>::V; ++i) Bs[idx_halves<N>(i, t.h) * Geo<N>::RS + t.q] = x[i];
 }
 
 // Bs -> the row pair's packed spectrum (k3 in PARITY); its inverse transform
 // has the reals of row q in x.x, of row q + N/2 in x.y (i3 in HALVES)
 template <int N>
 __device__ __forceinline__ void load_rows(ci64 (&x)[Geo<N>::V], const PlaneThread& t, const ci64* Bs) {
-  constexpr int HC = Geo<N>::HC, V = Geo<N>::V;
-  const ci64* ra = Bs + t.q * HC;
-  const ci64* rb = ra + (N / 2) * HC;
+  constexpr int RS = Geo<N>::RS, V = Geo<N>::V;
+  const ci64* ra = Bs + t.q * RS;
+  const ci64* rb = ra + (N / 2) * RS;
   if constexpr (Geo<N>::T == 1) {
     const ci64 a0 = ra[0], b0 = rb[0];  // (x_0, x_(N/2)) of each row
     x[0] = ci64{a0.x, b0.x};
@@ -670,8 +694,8 @@ __device__ __forceinline__ void load_rows(ci64 (&x)[Geo<N>::V], const PlaneThrea
 // pair's own slots of Bs: k < N/2 in row q, the others in row q + N/2
 template <int N>
 __device__ __forceinline__ void store_rows(const ci64 (&x)[Geo<N>::V], const PlaneThread& t, ci64* Bs) {
-  ci64* ra = Bs + t.q * Geo<N>::HC;
-  ci64* rb = ra + (N / 2) * Geo<N>::HC;
+  ci64* ra = Bs + t.q * Geo<N>::RS;
+  ci64* rb = ra + (N / 2) * Geo<N>::RS;
 #pragma unroll
   for (int i = 0; i < Geo<N>::V; ++i)
     (i < Geo<N>::V / 2 ? ra : rb)[idx_parity<N>(i, t.h) % (N / 2)] = ci64{x[i].y, x[i].x};
@@ -681,12 +705,12 @@ __device__ __forceinline__ void store_rows(const ci64 (&x)[Geo<N>::V], const Pla
 // twice its value, from z(q) and z(N - q) of every row pair
 template <int N>
 __device__ __forceinline__ void load_columns(ci64 (&x)[Geo<N>::V], const PlaneThread& t, const ci64* Bs) {
-  constexpr int HC = Geo<N>::HC, V = Geo<N>::V;
+  constexpr int RS = Geo<N>::RS, V = Geo<N>::V;
   const bool packed = t.q == 0;
 #pragma unroll
   for (int i = 0; i < V / 2; ++i) {
     const int r = Geo<N>::T == 1 ? i : t.h * (V / 2) + i;
-    const ci64 z1 = Bs[r * HC + t.q], z2 = Bs[(r + N / 2) * HC + (packed ? 0 : N / 2 - t.q)];
+    const ci64 z1 = Bs[r * RS + t.q], z2 = Bs[(r + N / 2) * RS + (packed ? 0 : N / 2 - t.q)];
     x[i] = packed ? ci64{z2.x, z1.x} : ci64{z1.y - z2.y, z1.x + z2.x};
     x[V / 2 + i] = packed ? ci64{z2.y, z1.y} : ci64{z2.x - z1.x, z1.y + z2.y};
   }
@@ -723,25 +747,18 @@ __device__ __forceinline__ double plane_bound(float top, int E, int s) { return 
 // of its entries' values.
 // grid = (N / PPC, J, B), block = Planes<N, PPC>::THREADS.
 template <int N, int PPC>
-__global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_plane(ci64* __restrict__ W, const int* __restrict__ EA,
+__global__ void __launch_bounds__(Planes<N, PPC>::THREADS, Planes<N, PPC>::BLOCKS) k_plane(ci64* __restrict__ W, const int* __restrict__ EA,
                                                                  const i64* __restrict__ mh,
-                                                                 const int* __restrict__ me, int* __restrict__ EP,
+                                                                 const int* __restrict__ em, int* __restrict__ EP,
                                                                  double* __restrict__ BP) {
   constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, V = Geo<N>::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned red[4 * PPC];
-  __shared__ int me3[N];       // exponent distances of M^h along axis 3
-  __shared__ float scale3[N];  // 2^-me3
   const PlaneThread t = plane_thread<N>(threadIdx.x);
   const int j = blockIdx.y, b = blockIdx.z, i1 = blockIdx.x * PPC + t.pp;
   const size_t u = (size_t)b * gridDim.y + j;
-  ci64* Bs = (ci64*)smem_raw + (size_t)t.pp * NC;
+  ci64* Bs = (ci64*)smem_raw + (size_t)t.pp * N * Geo<N>::RS;
   ci64* gw = W + (u * N + i1) * NC;
-  me += b * 3 * N;
-  for (int i = threadIdx.x; i < N; i += Planes<N, PPC>::THREADS) {
-    me3[i] = me[2 * N + i];
-    scale3[i] = exp2_neg(me3[i]);
-  }
   if (threadIdx.x < 4 * PPC) red[threadIdx.x] = 0;
   __syncthreads();
   int E = EA[u], s = 0;
@@ -750,28 +767,33 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_plane(ci64* __restr
 #pragma unroll 1
   for (int pass = 0; pass < 4; ++pass) {
     if (pass == 2) {
-      // x M^h: the products (parts exchanged from here on), their pencil sum,
-      // and one shift of each value by its own exponent distance and the plane's
+      // x M^h (parts exchanged from here on).  psi_j is largest in the tails,
+      // where M^h is smallest, so the products are far below the product of
+      // the largest values; they are formed with as many more bits as a bound
+      // of their own pencil sum leaves room for.  Without these the products'
+      // rounding drowned the result (25 times the error in the 2-norm).
       const i64* mp = mh + ((size_t)b * N + i1) * N * N + t.q;
-      const int mea = me[N + t.q], meb = me[N + N / 2 + t.q];
-      float sa = 0.f, sb = 0.f;
+      float sum = 0.f;
 #pragma unroll
       for (int i = 0; i < V; ++i) {
-        const int i3 = idx_halves<N>(i, t.h);
-        x[i] = ci64{mul(x[i].y, unpack_mult(__ldg(mp + i3 * N + N / 2))), mul(x[i].x, unpack_mult(__ldg(mp + i3 * N)))};
-        sa += fabsf((float)(int)(x[i].y >> 32)) * scale3[i3];
-        sb += fabsf((float)(int)(x[i].x >> 32)) * scale3[i3];
+        const i64* m = mp + idx_halves<N>(i, t.h) * N;
+        sum += (fabsf((float)(int)(x[i].x >> 32)) + 1.f) * (float)((int)(__ldg(m) >> 32) + 1);
+        sum += (fabsf((float)(int)(x[i].y >> 32)) + 1.f) * (float)((int)(__ldg(m + N / 2) >> 32) + 1);
       }
-      sa = (sa * exp2_neg(mea) + sb * exp2_neg(meb)) * 1.00002f + (float)(2 * V);
-      s = shift_for(plane_max<N>(pencil_sum<N>(sa), red + 2 * PPC + t.pp), kSumBits);
-      const int da = mea + s, db = meb + s;
+      sum = sum * (1.00002f * 0x1p-33f) + 1.f;  // of the products / 2^64, in units of 2^32
+      s = shift_for(plane_max<N>(pencil_sum<N>(sum), red + 2 * PPC + t.pp), kSumBits);
+      const int bits = min(max(-s, 1), 31);
 #pragma unroll
       for (int i = 0; i < V; ++i) {
-        const int d = me3[idx_halves<N>(i, t.h)];
-        x[i] = ci64{shift_any(x[i].x, d + db), shift_any(x[i].y, d + da)};
+        const i64* m = mp + idx_halves<N>(i, t.h) * N;
+        x[i] = ci64{mul_finer(x[i].y, __ldg(m + N / 2), bits), mul_finer(x[i].x, __ldg(m), bits)};
       }
-      E += 64 + me[i1] + s;
-      s = 0;
+      E += 64 + em[b * N + i1] - bits;
+      s += bits;
+      if (s > 0) {  // one bit was too many
+        shift_all<V>(x, s);
+        E += s;
+      }
     } else {
       if (pass == 0) {
 #pragma unroll
@@ -785,7 +807,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_plane(ci64* __restr
       } else {
         load_columns<N>(x, t, Bs);
       }
-      top = normalise<N>(x, s, E, red + pass * PPC + t.pp);
+      top = normalise<N>(x, s, E, red + pass * PPC + t.pp, pass == 3);
     }
     pencil_inverse<N>(x, t.h, pass < 2);
     if (pass == 0) {
@@ -836,7 +858,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
   const PlaneThread t = plane_thread<N>(threadIdx.x);
   const int b = blockIdx.y, i1 = blockIdx.x * PPC + t.pp;
   const size_t u = (size_t)blockIdx.z * gridDim.y + b;
-  ci64* Bs = (ci64*)smem_raw + (size_t)t.pp * NC;
+  ci64* Bs = (ci64*)smem_raw + (size_t)t.pp * N * Geo<N>::RS;
   double* D = (double*)Bs;  // [i2][i3], row stride N + 1
   const bool ratio = with_ratio && blockIdx.z == 0;
   if (threadIdx.x < 3 * PPC) red[threadIdx.x] = 0;
@@ -879,7 +901,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
     } else {
       load_columns<N>(x, t, Bs);
     }
-    sum = normalise<N>(x, s, E, red + (1 + pass) * PPC + t.pp);
+    sum = normalise<N>(x, s, E, red + (1 + pass) * PPC + t.pp, true);
     pencil_inverse<N>(x, t.h, false);
     if (pass == 0) {
       plane_sync<N>();  // D has been read
@@ -1089,8 +1111,8 @@ __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict
   }
   __syncthreads();
   for (int e = threadIdx.x; e < J * N; e += 32 * WARPS) {
-    const int d = el + q[e / N] - 64 - EP[(size_t)b * J * N + e];
-    sp[e] = d > 63 ? 63 : (d < -63 ? -63 : d);
+    // >= 0: BP is at least 2^60 of its plane's units
+    sp[e] = min(max(el + q[e / N] - 64 - EP[(size_t)b * J * N + e], 0), 63);
   }
   __syncthreads();
   ci64* acc = (ci64*)smem_raw + w * V * 32 + lane;
@@ -1107,7 +1129,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict
 #pragma unroll
     for (int i = 0; i < V; ++i) {
       const int s = su[idx_parity<N>(i, h)];
-      x[i] = ci64{shift_any(x[i].x, s), shift_any(x[i].y, s)};
+      x[i] = ci64{shift_right(x[i].x, s), shift_right(x[i].y, s)};
     }
     dft_time<N, false>(x, h);
 #pragma unroll
@@ -1172,7 +1194,7 @@ __global__ void __launch_bounds__(Combine<N, PPC, MODE>::THREADS)
   const int fl = threadIdx.x / C::GROUP, f = C::F0 + fl;
   const PlaneThread t = plane_thread<N>(threadIdx.x % C::GROUP);
   const int B = gridDim.y, b = blockIdx.y, i1 = blockIdx.x * PPC + t.pp;
-  ci64* Bs = (ci64*)smem_raw + (size_t)(fl * PPC + t.pp) * NC;
+  ci64* Bs = (ci64*)smem_raw + (size_t)(fl * PPC + t.pp) * N * Geo<N>::RS;
   for (int i = threadIdx.x; i < 3 * C::FIELDS * PPC; i += C::THREADS) red[i] = 0;
   if constexpr (C::MAXW) {
     for (int i = threadIdx.x; i < 3 * N; i += C::THREADS) em[i] = inst[(size_t)b * Inst<N>::SIZE + Inst<N>::EM + i];
@@ -1221,7 +1243,7 @@ __global__ void __launch_bounds__(Combine<N, PPC, MODE>::THREADS)
       E += sc;
     } else {
       load_rows<N>(x, t, Bs);
-      normalise<N>(x, s, E, slot + 2 * PPC);
+      normalise<N>(x, s, E, slot + 2 * PPC, true);
     }
     pencil_inverse<N>(x, t.h, true);
     if (pass == 0) {
@@ -1231,8 +1253,8 @@ __global__ void __launch_bounds__(Combine<N, PPC, MODE>::THREADS)
   }
   plane_sync<N>();
   // the field as FP64 (u already times M) in the rows' own slots of Bs
-  double* ra = (double*)(Bs + t.q * HC);
-  double* rb = (double*)(Bs + (t.q + N / 2) * HC);
+  double* ra = (double*)(Bs + t.q * Geo<N>::RS);
+  double* rb = (double*)(Bs + (t.q + N / 2) * Geo<N>::RS);
 #pragma unroll
   for (int i = 0; i < V; ++i) {
     const int i3 = idx_halves<N>(i, t.h);
@@ -1249,8 +1271,8 @@ __global__ void __launch_bounds__(Combine<N, PPC, MODE>::THREADS)
   const bool nan = MODE != FACTOR && bad[b] != 0;
   for (int e = threadIdx.x; e < PPC * N * N; e += C::THREADS) {
     const int i3 = e % N, r = e / N;  // row r of the block's planes
-    const double* v = (const double*)((ci64*)smem_raw + (size_t)r * HC) + i3;
-    constexpr size_t FS = (size_t)PPC * NC * 2;  // doubles from one field's planes to the next
+    const double* v = (const double*)((ci64*)smem_raw + (size_t)r * Geo<N>::RS) + i3;
+    constexpr size_t FS = (size_t)PPC * N * Geo<N>::RS * 2;  // doubles from one field's planes to the next
     double y = v[0];
     if constexpr (MODE == QUAD) y = y - g[o + e] * v[FS];
     if constexpr (C::MAXW) y = y - v[FS] - (MODE == CACHED ? wc[o + e] : v[2 * FS]) * g[o + e];

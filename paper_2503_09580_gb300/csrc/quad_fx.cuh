@@ -25,7 +25,7 @@ struct GeoQ {
   static constexpr bool WARP = TPP == 16 || TPP == 32;
   static constexpr int PPC = WARP ? 32 / TPP * 2 : (TPP == 24 ? 4 : 1);  // planes per block
   static constexpr int THREADS = TPP * PPC;
-  static constexpr int RS = N + 1;  // odd row stride of the exchange buffer
+  static constexpr int RS = T == 2 ? N + 2 : N + 1;  // row stride of the exchange buffer (Geo::RS)
   static constexpr size_t BYTES = (size_t)PPC * (sizeof(ci64) * N * RS + sizeof(i64) * N * N);
 };
 
