@@ -49,6 +49,7 @@ struct lbo_plan {
   const double* mc_params = nullptr;
   int mc_batch = 0, mc_precision = -1, mc_path = -1;
   bool mc_valid = false;
+  double mc_eps = 0;  // cut-off level of the cached tables (fixed-point form of FP64)
   void *mc_uh = nullptr, *mc_w = nullptr;
   size_t mc_uh_bytes = 0, mc_w_bytes = 0;
   // workspace of the generic path

@@ -42,6 +42,12 @@ struct Geo {
   static constexpr bool WARP = TPP == 8 || TPP == 16 || TPP == 32;
 };
 
+// The axis-1 frequencies |k| in BANDS bands, [0, N/2) in quarters and N/2: the
+// magnitudes of r^ and of u^_j that bound their products' pencil sums.
+constexpr int BANDS = 5;
+template <int N>
+__device__ __forceinline__ constexpr int band(int k) { return k / (N / 8); }
+
 constexpr int kSumBits = 60;       // sum(|re| + |im|) of a pencil before its transform, at most 2^60
 constexpr int kZeroExp = -100000;  // exponent of an all-zero column
 
@@ -324,7 +330,8 @@ __global__ void __launch_bounds__(256) k_mh(const double* __restrict__ inst, con
 
 // ------------------------------------------------------------ u^_j
 // One unit's octant U[u][k1][k2][k3] 2^eU[u] = FFT(M^g phit_j), scaled to a
-// largest entry in [2^61, 2^62): the weight in FP64 as k_uhat_planes forms it,
+// largest entry in [2^61, 2^62), and ub[u][band][k2][k3], its largest magnitude
+// over a band of k1 times 2^-62: the weight in FP64 as k_uhat_planes forms it,
 // then the three DCT-I passes, each after a shift by its own largest pencil
 // sum.  One thread per pencil, the octant in shared memory; at N = 64, where
 // that takes 287 KB, a cluster of two blocks holds half of the planes d1 each
@@ -388,7 +395,8 @@ __device__ __forceinline__ void dct_shifted(i64 (&x)[H + 1], int s) {  // the sh
 template <int N>
 __global__ void __launch_bounds__(Octant<N>::BLOCK) k_uhat(const double* __restrict__ inst,
                                                          const double* __restrict__ phit, i64* __restrict__ U,
-                                                         int* __restrict__ eU, int* __restrict__ bad, int J) {
+                                                         int* __restrict__ eU, float* __restrict__ ub,
+                                                         int* __restrict__ bad, int J) {
   using O = Octant<N>;
   constexpr int H = N / 2, HC = O::HC, HC2 = O::HC2, HC3 = O::HC3, CL = O::CL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -460,8 +468,15 @@ __global__ void __launch_bounds__(Octant<N>::BLOCK) k_uhat(const double* __restr
   const int l = m ? __clz(m) - 1 : 0;  // left shift to a top bit of 2^61
   if (on) {
     i64* dst = U + u * HC3 + q;
+    unsigned top[BANDS] = {};
 #pragma unroll
-    for (int d = 0; d < HC; ++d) dst[d * HC2] = (i64)((u64)x[d] << l);
+    for (int d = 0; d < HC; ++d) {
+      const i64 v = (i64)((u64)x[d] << l);
+      dst[d * HC2] = v;
+      top[band<N>(d)] = max(top[band<N>(d)], (unsigned)((v ^ (v >> 63)) >> 32));
+    }
+#pragma unroll
+    for (int d = 0; d < BANDS; ++d) ub[(u * BANDS + d) * HC2 + q] = ((float)top[d] + 1.f) * (1.00001f * 0x1p-30f);
   }
   if (t == 0 && rank == 0) eU[u] = E - l;
 }
@@ -469,9 +484,10 @@ __global__ void __launch_bounds__(Octant<N>::BLOCK) k_uhat(const double* __restr
 // ------------------------------------------------------------ exponents
 // EA[u]: the exponent of the products u^_j r^ of unit u, such that
 // sum(|re| + |im|) over every axis-1 pencil is at most 2^60; from the largest
-// sum_k1 |U| rm over the columns (rm of k_axis1_head).  grid = (J, B), block = 256.
+// sum over the bands of ub (k_uhat) times rm (k_axis1_head) over the columns.
+// grid = (J, B), block = 256.
 template <int N>
-__global__ void __launch_bounds__(256) k_unit_scale(const i64* __restrict__ U, const int* __restrict__ eU,
+__global__ void __launch_bounds__(256) k_unit_scale(const float* __restrict__ ub, const int* __restrict__ eU,
                                                     const float* __restrict__ rm, const int* __restrict__ eR,
                                                     int* __restrict__ EA, int J) {
   constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC;
@@ -493,12 +509,11 @@ __global__ void __launch_bounds__(256) k_unit_scale(const i64* __restrict__ U, c
   float f = 0.f;
   for (int c = t; c < NC; c += 256) {
     const int k2 = c / HC, k3 = c % HC, a2 = k2 <= N / 2 ? k2 : N - k2;
-    const float* r = rm + (size_t)b * HC * NC + c;
-    const i64* uc = U + u * HC * HC * HC + a2 * HC + k3;
+    const float* r = rm + (size_t)b * BANDS * NC + c;
+    const float* uc = ub + u * BANDS * HC * HC + a2 * HC + k3;
     float s = 0.f;
 #pragma unroll
-    for (int k = 0; k < HC; ++k)
-      s += (fabsf((float)(int)(uc[(size_t)k * HC * HC] >> 32)) + 1.f) * 0x1p-30f * r[(size_t)k * NC];
+    for (int k = 0; k < BANDS; ++k) s += uc[(size_t)k * HC * HC] * r[(size_t)k * NC];
     const int d = et - eR[b * NC + c];
     if (d < 120) f = fmaxf(f, s * __uint_as_float((unsigned)(127 - d) << 23));
   }
@@ -872,8 +887,10 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
   __syncthreads();
   const double* g = field + ((size_t)b * N + i1) * N * N;
   unsigned top = 0;
-  for (int e = t.tp; e < N * N; e += TPP) {
-    const int i3 = e % N, i2 = e / N;
+  // the loads of several points in flight: one at a time took 10 of 20 us for a single instance
+#pragma unroll 8
+  for (int it = 0; it < N * N / TPP; ++it) {
+    const int e = t.tp + it * TPP, i3 = e % N, i2 = e / N;
     double v = g[e];
     if (ratio) {
       const bool cut = cutoff && __dadd_rn(__dadd_rn(sq[i1], sq[N + i2]), sq[2 * N + i3]) >= dstar;
@@ -941,8 +958,8 @@ __device__ __forceinline__ unsigned top_bits(const ci64 (&x)[V]) {  // bits 31..
 }
 
 // Axis 1 of the head, one column per pencil.  z = 0: r^ = FFT_1 of F[0], every
-// column scaled to a top bit of 2^61 with its exponent eR; rm[b][k][col], k =
-// 0..N/2: (|R(k)|_1 + |R(-k)|_1) 2^-62 (k_unit_scale), once for k = 0, N/2.  z = 1: F[1] <- InvFFT_1(FFT_1(F[src1]) omega) (src1 = 1: in
+// column scaled to a top bit of 2^61 with its exponent eR; rm[b][band][col]:
+// sum of (|re| + |im|) 2^-62 over the band's |k1| (k_unit_scale).  z = 1: F[1] <- InvFFT_1(FFT_1(F[src1]) omega) (src1 = 1: in
 // place).  z = 2: F[2] = InvFFT_1(FFT(M) omega), FFT(M) from its factors.  Of
 // F[1], F[2] every column has its exponent EC[z][b][col].  z0: the first z of
 // the launch.  omega: multipliers indexed by |k|^2, or with omega3 by the
@@ -1005,29 +1022,25 @@ __global__ void __launch_bounds__(64) k_axis1_head(ci64* __restrict__ F, const i
     if (T == 2) m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
     const int l = m ? __clz(m) - 1 : 0;
     ci64* dst = R + (size_t)b * N * NC + col;
-    float* rc = rm + (size_t)b * HC * NC + col;
-    float mag[V];
+    float sums[BANDS] = {};
 #pragma unroll
     for (int i = 0; i < V; ++i) {
       const ci64 v = ci64{(i64)((u64)x[i].x << l), (i64)((u64)x[i].y << l)};
       if (on) dst[(size_t)idx_halves<N>(i, h) * NC] = v;
-      mag[i] = (fabsf((float)(int)(v.x >> 32)) + fabsf((float)(int)(v.y >> 32)) + 2.f) * 0x1p-30f;
-    }
-    // k and N - k: in one thread, or value i of a thread with value V - i of the other
-#pragma unroll
-    for (int i = 0; i <= N / 2 / T; ++i) {
-      float w = mag[i];
+      const float w = (fabsf((float)(int)(v.x >> 32)) + fabsf((float)(int)(v.y >> 32)) + 2.f) * 0x1p-30f;
       if (T == 1) {
-        if (i > 0 && i < N / 2) w += mag[N - i];
-        if (on) rc[(size_t)i * NC] = w;
-      } else if (i == 0) {
-        if (h == 1) w += mag[V / 2];
-        if (on) rc[(size_t)(h * (V / 2)) * NC] = w;
-        if (on && h == 0) rc[(size_t)(N / 2) * NC] = mag[V / 2];
-      } else if (i < V / 2) {
-        w += __shfl_xor_sync(0xffffffffu, mag[V - i], 1);
-        if (on) rc[(size_t)(h * (V / 2) + i) * NC] = w;
+        sums[band<N>(i <= N / 2 ? i : N - i)] += w;
+      } else {  // |k| of value i of thread 0, 1: i, N/4 + i below, N/2 - i, N/4 - i above N/2
+        constexpr int Q = N / 4;
+        const float w0 = h ? 0.f : w, w1 = h ? w : 0.f;
+        sums[band<N>(i < Q ? i : (i == Q ? N / 2 : N / 2 - (i - Q)))] += w0;
+        sums[band<N>(i < Q ? Q + i : Q - (i - Q))] += w1;
       }
+    }
+#pragma unroll
+    for (int d = 0; d < BANDS; ++d) {
+      const float w = pencil_sum<N>(sums[d]);
+      if (on && h == 0) rm[((size_t)b * BANDS + d) * NC + col] = w;
     }
     if (!on) return;
     if (h == 0) eR[b * NC + col] = m ? E - l : kZeroExp;
@@ -1269,6 +1282,7 @@ __global__ void __launch_bounds__(Combine<N, PPC, MODE>::THREADS)
   __syncthreads();
   const size_t o = ((size_t)b * N + blockIdx.x * PPC) * N * N;
   const bool nan = MODE != FACTOR && bad[b] != 0;
+#pragma unroll 4
   for (int e = threadIdx.x; e < PPC * N * N; e += C::THREADS) {
     const int i3 = e % N, r = e / N;  // row r of the block's planes
     const double* v = (const double*)((ci64*)smem_raw + (size_t)r * Geo<N>::RS) + i3;

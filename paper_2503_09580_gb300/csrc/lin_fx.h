@@ -21,8 +21,13 @@ struct Tables {
 struct Cache {
   const long long* U;  // [B][J][(N/2+1)^3] u^_j
   const int* eU;       // [B][J] its exponents
+  const float* ub;     // [B][J][BANDS][(N/2+1)^2] its magnitudes (lin_fx.cuh)
   const int* bad;      // [B] 1: not finite
+  const double* inst;  // the instances' tables (lin_fx.cuh) for the cut-off level eps
+  const int* em;
+  const long long* mh;
   const double* w;     // [B][N^3] InvFFT(FFT(M) omega)
+  double eps;
 };
 
 // The hemisphere rule of Q(f,f) on the device, and optionally the loss

@@ -15,7 +15,9 @@ namespace fx {
   size_t workspace_bytes_##n(int B, int G, int J, bool own_u);                                                    \
   lbo_status apply_##n(lbo_plan* p, const Tables& tb, const double* params, const double* g, double* out, int B,  \
                        int G, void* ws, const Cache* mc);                                                         \
-  lbo_status precompute_##n(lbo_plan* p, const Tables& tb, const double* params, int B, void* ws, const Cache& mc);
+  lbo_status precompute_##n(lbo_plan* p, const Tables& tb, const double* params, int B, void* ws, const Cache& mc); \
+  size_t cache_bytes_##n(int B, int J);                                                                           \
+  Cache cache_at_##n(void* base, int B, int J, int b0);
 #define LBO_FX_QDECL(n)                                                                                            \
   size_t q_workspace_bytes_##n(int B, int J, int M, bool position);                                               \
   lbo_status q_apply_##n(lbo_plan* p, const Tables& tb, const QuadRule& rule, const double* f, double* out, int B, \
@@ -86,18 +88,29 @@ int part_size(const lbo_plan* p, int B) {
   return std::min(B, most);
 }
 
-size_t octant(const lbo_plan* p) {
-  const size_t hc = p->N / 2 + 1;
-  return hc * hc * hc;
+size_t cache_bytes(int N, int B, int J) {
+  switch (N) {
+    case 16: return cache_bytes_16(B, J);
+    case 24: return cache_bytes_24(B, J);
+    case 32: return cache_bytes_32(B, J);
+    case 48: return cache_bytes_48(B, J);
+    default: return cache_bytes_64(B, J);
+  }
 }
 
-// The cache buffer p->mc_uh holds U, eU and the flags; p->mc_w the loss factor.
+// The cache of B instances (p->mc_uh; the loss factor in p->mc_w) from instance b0 on.
 Cache cache_at(const lbo_plan* p, int B, int b0) {
-  const size_t n3 = (size_t)p->N * p->N * p->N;
-  const long long* U = (const long long*)p->mc_uh;
-  const int* eU = (const int*)(U + (size_t)B * p->J * octant(p));
-  return Cache{U + (size_t)b0 * p->J * octant(p), eU + (size_t)b0 * p->J, eU + (size_t)B * p->J + b0,
-               (const double*)p->mc_w + (size_t)b0 * n3};
+  Cache c;
+  switch (p->N) {
+    case 16: c = cache_at_16(p->mc_uh, B, p->J, b0); break;
+    case 24: c = cache_at_24(p->mc_uh, B, p->J, b0); break;
+    case 32: c = cache_at_32(p->mc_uh, B, p->J, b0); break;
+    case 48: c = cache_at_48(p->mc_uh, B, p->J, b0); break;
+    default: c = cache_at_64(p->mc_uh, B, p->J, b0);
+  }
+  c.w = (const double*)p->mc_w + (size_t)b0 * p->N * p->N * p->N;
+  c.eps = p->mc_eps;
+  return c;
 }
 
 // Multipliers value 2^-exponent of n doubles, largest in [2^61, 2^62).
@@ -183,9 +196,7 @@ lbo_status q_apply_part(lbo_plan* p, const Tables& tb, const QuadRule& rule, con
 }  // namespace
 }  // namespace fx
 
-size_t fx_cache_bytes(const lbo_plan* p, int B) {
-  return (size_t)B * p->J * (fx::octant(p) * sizeof(long long) + sizeof(int)) + sizeof(int) * (size_t)B;
-}
+size_t fx_cache_bytes(const lbo_plan* p, int B) { return fx::cache_bytes(p->N, B, p->J); }
 
 void free_fx_tables(lbo_plan* p) {
   if (p->d_fx) cudaFree(p->d_fx);
@@ -217,6 +228,7 @@ lbo_status precompute_fx(lbo_plan* p, const double* params, int B) {
   if (st != LBO_OK) return st;
   cudaError_t e = cudaMemsetAsync((void*)fx::cache_at(p, B, 0).bad, 0, sizeof(int) * (size_t)B, p->stream);
   if (e != cudaSuccess) return cuda_fail(e, "fixed-point flags");
+  p->mc_eps = p->eps;
   p->last_launches = 0;
   for (int b0 = 0; b0 < B && st == LBO_OK; b0 += part)
     st = fx::precompute_part(p, tb, params + 5 * (size_t)b0, std::min(part, B - b0), fx::cache_at(p, B, b0));

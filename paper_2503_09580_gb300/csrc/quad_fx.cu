@@ -19,7 +19,7 @@ namespace fx {
 namespace {
 
 constexpr int N = LBO_FX_N;
-constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, T = Geo<N>::T;
+constexpr int NC = Geo<N>::NC, T = Geo<N>::T;
 constexpr size_t H = (size_t)N * NC, n3 = (size_t)N * N * N;
 constexpr int ACC_WARPS = 8, PPC = PlanesPPC<N>::v, CPPC = CombinePPC<N>::v;
 
@@ -59,7 +59,7 @@ struct Buffers {
     take(om3, position ? H : 0);
     take(BPh, B * N);
     take(BP, c.G * J * N);
-    take(rm, B * HC * NC);
+    take(rm, B * BANDS * NC);
     take(eR, B * NC);
     take(EF, B);
     take(EPh, B * N);

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_q_position_multipliers(const double* __
 template <int N>
 __global__ void __launch_bounds__(64) k_q_rescale(ci64* __restrict__ R, const int* __restrict__ eR,
                                                   const float* __restrict__ rm, int* __restrict__ EF) {
-  constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC;
+  constexpr int NC = Geo<N>::NC;
   __shared__ int top;
   const int b = blockIdx.y, col = blockIdx.x * 64 + threadIdx.x;
   if (threadIdx.x == 0) top = kZeroExp;
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(64) k_q_rescale(ci64* __restrict__ R, const in
   int e = kZeroExp;
   for (int c = threadIdx.x; c < NC; c += 64) {
     float s = 0x1p-30f;
-    for (int k = 0; k < HC; ++k) s += rm[((size_t)b * HC + k) * NC + c];  // 2^-62 of the pencil's sum
+    for (int k = 0; k < BANDS; ++k) s += rm[((size_t)b * BANDS + k) * NC + c];  // 2^-62 of the pencil's sum
     if (eR[b * NC + c] != kZeroExp) e = max(e, eR[b * NC + c] + ilogbf(s * 1.0001f) + 1);
   }
   e = __reduce_max_sync(0xffffffffu, e);
