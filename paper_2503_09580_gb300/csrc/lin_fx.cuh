@@ -5,7 +5,7 @@
 // A unit u = (instance b, radial node j) is one pass psi_j = InvFFT(u^_j r^),
 // psi^_j = FFT(M^h psi_j).  All units of a group of instances run in one
 // launch per kernel, so a single instance still fills the chip with its J
-// nodes, and a group is chosen so that its half spectra stay in the L2 cache:
+// nodes:
 //
 //   k_instance       per-instance tables (all exponentials)
 //   k_mh             the table of M^h, the 1-D transforms of M's factors
