@@ -13,6 +13,7 @@ namespace {
 
 constexpr int RED_BLOCKS = 304;  // 2 x 152 SMs
 constexpr int RED_THREADS = 256;
+constexpr int WALL_BLOCKS = 16;
 constexpr int DOT_TILE = 8;
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
@@ -46,18 +47,29 @@ __global__ void __launch_bounds__(RED_THREADS) k_dots(const double* __restrict__
     }
 #pragma unroll
     for (int t = 0; t < DOT_TILE; ++t) {
+      if (k0 + t >= K) break;
       double s = block_sum(acc[t], sh);
-      if (threadIdx.x == 0 && k0 + t < K) part[blockIdx.x * K + k0 + t] = s;
+      if (threadIdx.x == 0) part[blockIdx.x * K + k0 + t] = s;
     }
   }
 }
 
-// out[k] = sum_b part[b*K + k] (fixed order: deterministic)
+// sum_b part[b*K + k] by one warp, in a fixed order (deterministic); valid in
+// every lane.  One thread's chain of RED_BLOCKS loads and additions took 15 of
+// the 22 us of a launch.
+__device__ __forceinline__ double warp_sum_parts(const double* __restrict__ part, int nb, int K, int k) {
+  double s = 0;
+#pragma unroll 10
+  for (int b = threadIdx.x & 31; b < nb; b += 32) s += part[(size_t)b * K + k];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// out[k] = sum_b part[b*K + k], one warp per k
 __global__ void k_reduce_parts(const double* __restrict__ part, int nb, int K, double* __restrict__ out) {
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    double s = 0;
-    for (int b = 0; b < nb; ++b) s += part[b * K + k];
-    out[k] = s;
+  for (int k = threadIdx.x >> 5; k < K; k += blockDim.x >> 5) {
+    const double s = warp_sum_parts(part, nb, K, k);
+    if ((threadIdx.x & 31) == 0) out[k] = s;
   }
 }
 
@@ -128,37 +140,36 @@ __global__ void __launch_bounds__(512) k_cell_moments(const double* __restrict__
 }
 
 // res[0] = -kL h^3 sum v1^- v_1, res[1] = kR h^3 sum v1^+ v_nx (wall densities),
-// res[2] = dx h^3 sum v (total mass); blocks 0, 1 the walls, the rest the mass
+// res[2] = dx h^3 sum v (total mass): the blocks' shares, WALL_BLOCKS blocks for
+// each wall's cell (one block took 50 us for its 32^3 points) and the rest for
+// the mass; k_mass_finish adds them up
 __global__ void __launch_bounds__(RED_THREADS) k_wall_mass(const double* __restrict__ v, int N, int nx, double h,
-                                                           double dx, double kL, double kR,
-                                                           double* __restrict__ part, double* __restrict__ res) {
+                                                           double* __restrict__ part) {
   __shared__ double sh[32];
   const size_t n3 = (size_t)N * N * N, len = n3 * nx;
-  const double h3 = h * h * h;
-  if (blockIdx.x < 2) {
-    const double* x = v + (blockIdx.x == 0 ? 0 : (size_t)(nx - 1) * n3);
-    double a = 0;
-    for (size_t t = threadIdx.x; t < n3; t += blockDim.x) {
+  double a = 0;
+  if (blockIdx.x < 2 * WALL_BLOCKS) {
+    const int wall = blockIdx.x / WALL_BLOCKS, b = blockIdx.x % WALL_BLOCKS;
+    const double* x = v + (wall == 0 ? 0 : (size_t)(nx - 1) * n3);
+    for (size_t t = b * (size_t)blockDim.x + threadIdx.x; t < n3; t += (size_t)WALL_BLOCKS * blockDim.x) {
       const double v1 = (int(t / ((size_t)N * N)) - N / 2) * h;
-      a += (blockIdx.x == 0 ? fmin(v1, 0.0) : fmax(v1, 0.0)) * x[t];
+      a += (wall == 0 ? fmin(v1, 0.0) : fmax(v1, 0.0)) * x[t];
     }
-    double s = block_sum(a, sh);
-    if (threadIdx.x == 0) res[blockIdx.x] = blockIdx.x == 0 ? -kL * h3 * s : kR * h3 * s;
   } else {
-    double a = 0;
-    const int nb = gridDim.x - 2, b = blockIdx.x - 2;
+    const int nb = gridDim.x - 2 * WALL_BLOCKS, b = blockIdx.x - 2 * WALL_BLOCKS;
     for (size_t e = b * (size_t)blockDim.x + threadIdx.x; e < len; e += (size_t)nb * blockDim.x) a += v[e];
-    double s = block_sum(a, sh);
-    if (threadIdx.x == 0) part[b] = s;
   }
+  const double s = block_sum(a, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-__global__ void k_mass_finish(const double* __restrict__ part, int nb, double w, double* __restrict__ res) {
-  if (threadIdx.x == 0) {
-    double s = 0;
-    for (int b = 0; b < nb; ++b) s += part[b];
-    res[2] = w * s;
-  }
+// one warp each for the two walls and the mass; block = 96
+__global__ void k_mass_finish(const double* __restrict__ part, int nb, double wL, double wR, double w,
+                              double* __restrict__ res) {
+  const int q = threadIdx.x >> 5;
+  const double s = q < 2 ? warp_sum_parts(part + q * WALL_BLOCKS, WALL_BLOCKS, 1, 0)
+                         : warp_sum_parts(part + 2 * WALL_BLOCKS, nb, 1, 0);
+  if ((threadIdx.x & 31) == 0) res[q] = (q == 0 ? wL : (q == 1 ? wR : w)) * s;
 }
 
 // out = T v * cT + y * cY + e * m(v) * cE, T the upwind transport with
@@ -227,7 +238,7 @@ int grid_for(size_t len) {
 lbo_status dots(lbo_solver* S, const double* Vb, size_t ld, int K, const double* y, double* host_out) {
   cudaStream_t s = S->plan->stream;
   LBO_LAUNCH(S->plan, "solver_dots", s, k_dots, RED_BLOCKS, RED_THREADS, 0, Vb, ld, K, y, S->len, S->part);
-  LBO_LAUNCH(S->plan, "solver_reduce", s, k_reduce_parts, 1, 256, 0, S->part, RED_BLOCKS, K, S->res + 8);
+  LBO_LAUNCH(S->plan, "solver_reduce", s, k_reduce_parts, 1, 1024, 0, S->part, RED_BLOCKS, K, S->res + 8);
   cudaError_t e = cudaMemcpyAsync(host_out, S->res + 8, sizeof(double) * K, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return e == cudaSuccess ? LBO_OK : cuda_fail(e, "solver dots");
@@ -243,9 +254,10 @@ double norm2(lbo_solver* S, const double* y, lbo_status* st) {
 void wall_mass(lbo_solver* S, const double* v) {
   cudaStream_t s = S->plan->stream;
   const int nb = RED_BLOCKS;
-  LBO_LAUNCH(S->plan, "solver_wall_mass", s, k_wall_mass, nb + 2, RED_THREADS, 0, v, S->N, S->nx, S->h, S->dx,
-             S->kL, S->kR, S->part, S->res);
-  LBO_LAUNCH(S->plan, "solver_mass_finish", s, k_mass_finish, 1, 32, 0, S->part, nb, S->dx * S->h * S->h * S->h,
+  const double h3 = S->h * S->h * S->h;
+  LBO_LAUNCH(S->plan, "solver_wall_mass", s, k_wall_mass, nb + 2 * WALL_BLOCKS, RED_THREADS, 0, v, S->N, S->nx, S->h,
+             S->part);
+  LBO_LAUNCH(S->plan, "solver_mass_finish", s, k_mass_finish, 1, 96, 0, S->part, nb, -S->kL * h3, S->kR * h3, S->dx * h3,
              S->res);
 }
 
@@ -537,8 +549,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_dots_dev(const double* __restri
     }
 #pragma unroll
     for (int t = 0; t < DOT_TILE; ++t) {
+      if (k0 + t >= K) break;
       double s = block_sum(acc[t], sh);
-      if (threadIdx.x == 0 && k0 + t < K) part[blockIdx.x * K + k0 + t] = s;
+      if (threadIdx.x == 0) part[blockIdx.x * K + k0 + t] = s;
     }
   }
 }
@@ -548,9 +561,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_dots_dev(const double* __restri
 __global__ void k_reduce_h(const double* __restrict__ part, int nb, const int* __restrict__ ik, double* __restrict__ hv,
                            double* __restrict__ H, int m, int pass) {
   const int k = ik[IK_K], K = k + 1;
-  for (int i = threadIdx.x; i < K; i += blockDim.x) {
-    double s = 0;
-    for (int b = 0; b < nb; ++b) s += part[b * K + i];
+  for (int i = threadIdx.x >> 5; i < K; i += blockDim.x >> 5) {
+    const double s = warp_sum_parts(part, nb, K, i);
+    if ((threadIdx.x & 31) != 0) continue;
     hv[i] = s;
     H[(size_t)i * m + k] = pass == 0 ? s : H[(size_t)i * m + k] + s;
   }
@@ -558,11 +571,8 @@ __global__ void k_reduce_h(const double* __restrict__ part, int nb, const int* _
 
 // out = sqrt(sum of the parts)
 __global__ void k_norm_finish(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  if (threadIdx.x == 0) {
-    double s = 0;
-    for (int b = 0; b < nb; ++b) s += part[b];
-    *out = sqrt(s);
-  }
+  const double s = warp_sum_parts(part, nb, 1, 0);
+  if (threadIdx.x == 0) *out = sqrt(s);
 }
 
 // y -= sum_i c[i] V_i, i < *Kp + Kadd
@@ -705,7 +715,7 @@ lbo_status dev_iteration(lbo_solver* S, DevArnoldi* D, int in_graph) {
   for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, two passes, FP64
     LBO_LAUNCH(S->plan, "krylov_dots", s, k_dots_dev, RED_BLOCKS, RED_THREADS, 0, S->V, len, D->ik + IK_K, 1,
                S->w, len, S->part);
-    LBO_LAUNCH(S->plan, "krylov_reduce_h", s, k_reduce_h, 1, 256, 0, S->part, RED_BLOCKS, D->ik, D->hv, D->H, m,
+    LBO_LAUNCH(S->plan, "krylov_reduce_h", s, k_reduce_h, 1, 1024, 0, S->part, RED_BLOCKS, D->ik, D->hv, D->H, m,
                pass);
     LBO_LAUNCH(S->plan, "krylov_sub", s, k_sub_comb_dev, grid_for(len), 256, 0, S->w, S->V, len, D->ik + IK_K, 1,
                D->hv, len);
