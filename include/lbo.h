@@ -63,10 +63,12 @@ typedef enum {
                             throughout                                      */
   LBO_PREC_FP32 = 1,     /* FP32 transforms and products, FP64 in/out,
                             FP64 Maxwellians, cut-off and final combination */
-  LBO_PREC_FP32X2 = 2,   /* transforms and products in pairs of FP32 numbers
-                            (hi + lo, about 48 significant bits, FP32
-                            exponent range) on the FP32 pipe; FP64
-                            Maxwellians, ratio, cut-off and combination     */
+  LBO_PREC_FP32X2 = 2,   /* at least 48 significant bits in transforms and
+                            products; FP64 Maxwellians, ratio, cut-off and
+                            combination.  Default kernels: those of FP64
+                            (faster here and more accurate); LBO_OPT_KERNEL 1:
+                            pairs of FP32 numbers (hi + lo, FP32 exponent
+                            range) on the FP32 pipe                         */
   LBO_PREC_FP64X2 = 3,   /* transforms and products in pairs of FP64 numbers
                             (about 106 significant bits): the higher-
                             precision convolution of Sec. 3.4 (the paper

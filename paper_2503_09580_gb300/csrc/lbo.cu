@@ -293,11 +293,11 @@ static lbo_status dispatch_lin(lbo_plan* p, const double* params, const double* 
   return dispatch_generic<T>(p, plain_tables<T>(p), params, g, out, B, p->ws, cuh ? &mc : nullptr);
 }
 
-// kernel set of an apply call: 1 the fused FP32 kernels (N = 32), 2 FP64 in
-// fixed point on the integer pipe, 0 generic
+// kernel set of an apply call: 1 the fused FP32 kernels (N = 32), 2 fixed point
+// on the integer pipe (FP64 and FP32X2), 0 generic
 static int kernel_path(const lbo_plan* p) {
   if (p->kernel_choice != 0) return 0;
-  if (p->precision == LBO_PREC_FP64) return 2;
+  if (uses_fixed_point(p)) return 2;
   return p->precision == LBO_PREC_FP32 && p->N == 32 ? 1 : 0;
 }
 

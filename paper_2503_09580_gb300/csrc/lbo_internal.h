@@ -140,6 +140,14 @@ lbo_status precompute_twofold(lbo_plan* p, const double* params, int B, void* uh
 lbo_status twofold_tables(lbo_plan* p, const void** phi, const void** omega, const void** phit, const void** dct);
 void free_twofold_tables(lbo_plan* p);
 inline bool is_twofold_precision(int prec) { return prec == LBO_PREC_FP32X2 || prec == LBO_PREC_FP64X2; }
+// FP64 and FP32X2 run in 64-bit fixed point (lin_fx.cuh, quad_fx.cuh) unless
+// LBO_OPT_KERNEL asks for other kernels.  For FP32X2 that replaces pairs of
+// FP32 numbers, which are less accurate (48 bits) and slower: L at N = 32, batch
+// 256 takes 14.2 ms in pairs against 5.6, Q at N = 64, one instance, 32.8 ms
+// against 13.8.
+inline bool uses_fixed_point(const lbo_plan* p) {
+  return p->kernel_choice == 0 && (p->precision == LBO_PREC_FP64 || p->precision == LBO_PREC_FP32X2);
+}
 // bytes of one real number in the transform precision of the generic path
 inline size_t generic_real_bytes(int prec) { return prec == LBO_PREC_FP64X2 ? 16 : 8; }
 // split 16-bit precisions on the tensor cores (lin_dftmm.cu)

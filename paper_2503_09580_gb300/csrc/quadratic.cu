@@ -77,7 +77,8 @@ __global__ void k_to_transform_type(const double* __restrict__ a, T* __restrict_
 // The Eq. (2.16) multiplier in the plan's transform precision, rebuilt when
 // the precision, the hemisphere rule or the tables change.
 lbo_status ensure_omega_quadrature(lbo_plan* p, QuadState* qs) {
-  if (qs->d_omq && qs->omq_prec == p->precision && qs->omq_p == qs->p && qs->omq_tables == (const void*)p->d_phi64)
+  const int prec = uses_fixed_point(p) ? (int)LBO_PREC_FP64 : p->precision;  // fixed point converts it from FP64
+  if (qs->d_omq && qs->omq_prec == prec && qs->omq_p == qs->p && qs->omq_tables == (const void*)p->d_phi64)
     return LBO_OK;
   if (qs->d_omq) cudaFree(qs->d_omq);
   qs->d_omq = nullptr;
@@ -102,7 +103,7 @@ lbo_status ensure_omega_quadrature(lbo_plan* p, QuadState* qs) {
     }
   double2* d_fac = nullptr;
   double *d_w = nullptr, *d_out = nullptr;
-  const size_t rb = p->precision == LBO_PREC_FP32 ? 4 : generic_real_bytes(p->precision);
+  const size_t rb = prec == LBO_PREC_FP32 ? 4 : generic_real_bytes(prec);
   cudaError_t e = cudaMalloc(&d_fac, sizeof(double2) * fac.size());
   if (e == cudaSuccess) e = cudaMalloc(&d_w, sizeof(double) * wjm.size());
   if (e == cudaSuccess) e = cudaMalloc(&d_out, sizeof(double) * H);
@@ -119,7 +120,7 @@ lbo_status ensure_omega_quadrature(lbo_plan* p, QuadState* qs) {
       case 48: k_omega_quadrature<48><<<grid, 256, 0, p->stream>>>(d_fac, d_w, J * M, scale, d_out); break;
       default: k_omega_quadrature<64><<<grid, 256, 0, p->stream>>>(d_fac, d_w, J * M, scale, d_out); break;
     }
-    switch (p->precision) {
+    switch (prec) {
       case LBO_PREC_FP64:
         e = cudaMemcpyAsync(qs->d_omq, d_out, sizeof(double) * H, cudaMemcpyDeviceToDevice, p->stream);
         break;
@@ -138,7 +139,7 @@ lbo_status ensure_omega_quadrature(lbo_plan* p, QuadState* qs) {
     qs->d_omq = nullptr;
     return cuda_fail(e, "Eq. (2.16) loss multiplier");
   }
-  qs->omq_prec = p->precision;
+  qs->omq_prec = prec;
   qs->omq_p = qs->p;
   qs->omq_tables = p->d_phi64;
   return LBO_OK;
@@ -179,8 +180,8 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
   const size_t N = p->N, H = N * N * (N / 2 + 1), n3 = N * N * N;
   const int M = (int)qs->wm.size();
   const size_t rb = generic_real_bytes(p->precision);
-  // FP64 in fixed point on the integer pipe (quad_fx.cuh), its own buffers
-  const bool fixed = p->precision == LBO_PREC_FP64 && p->kernel_choice == 0;
+  // fixed point on the integer pipe (quad_fx.cuh), its own buffers
+  const bool fixed = uses_fixed_point(p);
   const size_t MB = fused || fixed ? 0 : (size_t)q_chunk(B, M, (int)N, rb);
   // FP64 at N = 32 (register kernels): the phase-factor table after the chunk buffers
   const size_t ptab = p->precision == LBO_PREC_FP64 && N == 32 && p->kernel_choice != 2
