@@ -89,8 +89,19 @@ FX_FN i64 mul(i64 y, Mult t) {
 FX_FN i64 mul_signed(i64 y, Mult t, int neg) {
   const unsigned yl = (unsigned)(u64)y;
   const int yh = (int)(y >> 32);
-  const int c = (int)(umulhi32(yl, (unsigned)t.th) - (yl & (unsigned)neg)) + mulhi32(yh, t.tl) + 1;
+  const int c = (int)(umulhi32(yl, (unsigned)t.th) - (yl & (unsigned)neg)) + mulhi32(yh, t.tl) + (int)(yl < 1u ? yl : 1u);
   return (i64)yh * t.th + (i64)c;
+}
+// round((y t + z w) / 2^64) for |y|, |z| <= 2^60 and a pair of multipliers whose
+// th have a norm of at most 2^30: the cross products together then stay below
+// 1.8 2^30.  Their four floors are balanced by 2 unless y = z = 0.
+FX_FN i64 mul_pair(i64 y, Mult t, i64 z, Mult w) {
+  const unsigned yl = (unsigned)(u64)y, zl = (unsigned)(u64)z, any = yl | zl;
+  const int yh = (int)(y >> 32), zh = (int)(z >> 32);
+  const int c = (int)(umulhi32(yl, (unsigned)t.th) - (yl & (unsigned)(t.th >> 31))) + mulhi32(yh, t.tl) +
+                (int)(umulhi32(zl, (unsigned)w.th) - (zl & (unsigned)(w.th >> 31))) + mulhi32(zh, w.tl) +
+                (int)(any < 2u ? any : 2u);
+  return (i64)yh * t.th + ((i64)zh * w.th + (i64)c);
 }
 // y m 2^(b - 64) for a multiplier 0 <= m < 2^60 split at bit 31 (pack_finer), 1 <= b
 // <= 31: b more bits than mul() keeps, all four partial products taken.

@@ -943,6 +943,10 @@ __device__ __forceinline__ SignedMult signed_mult(i64 y) {
   const Mult m = split_mult(y);
   return SignedMult{m, m.th >> 31};
 }
+__device__ __forceinline__ SignedMult signed_of(i64 packed) {
+  const Mult m = unpack_mult(packed);
+  return SignedMult{m, m.th >> 31};
+}
 // a z / 2^64 with a's parts as multipliers
 __device__ __forceinline__ ci64 cmul_mult(SignedMult ax, SignedMult ay, ci64 z) {
   return ci64{mul_signed(z.x, ax.m, ax.neg) - mul_signed(z.y, ay.m, ay.neg),

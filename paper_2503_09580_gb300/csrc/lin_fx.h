@@ -36,6 +36,9 @@ struct Cache {
 struct QuadRule {
   const double *gj, *sig, *wm;  // [J] radial nodes, [M][3] directions, [M] weights
   int M;
+  const int4* node;        // [M], ordered by class: (node, class, sigma_1 < 0, first of its class)
+  const int* class_begin;  // host, [classes + 1]: a class shares |sigma_1| and w_m
+  int classes;
   double wmax;
   const double* omega3;
   double omega3_bound;

@@ -19,7 +19,7 @@ namespace fx {
   size_t cache_bytes_##n(int B, int J);                                                                           \
   Cache cache_at_##n(void* base, int B, int J, int b0);
 #define LBO_FX_QDECL(n)                                                                                            \
-  size_t q_workspace_bytes_##n(int B, int J, int M, bool position);                                               \
+  size_t q_workspace_bytes_##n(int B, int J, const QuadRule& rule);                                             \
   lbo_status q_apply_##n(lbo_plan* p, const Tables& tb, const QuadRule& rule, const double* f, double* out, int B, \
                          void* ws);
 LBO_FX_QDECL(16)
@@ -174,13 +174,13 @@ lbo_status ensure(void** ws, size_t* have, size_t bytes) {
   return LBO_OK;
 }
 
-size_t q_workspace_bytes(int N, int B, int J, int M, bool position) {
+size_t q_workspace_bytes(int N, int B, int J, const QuadRule& rule) {
   switch (N) {
-    case 16: return q_workspace_bytes_16(B, J, M, position);
-    case 24: return q_workspace_bytes_24(B, J, M, position);
-    case 32: return q_workspace_bytes_32(B, J, M, position);
-    case 48: return q_workspace_bytes_48(B, J, M, position);
-    default: return q_workspace_bytes_64(B, J, M, position);
+    case 16: return q_workspace_bytes_16(B, J, rule);
+    case 24: return q_workspace_bytes_24(B, J, rule);
+    case 32: return q_workspace_bytes_32(B, J, rule);
+    case 48: return q_workspace_bytes_48(B, J, rule);
+    default: return q_workspace_bytes_64(B, J, rule);
   }
 }
 
@@ -244,7 +244,7 @@ lbo_status run_quadratic_fx(lbo_plan* p, const fx::QuadRule& rule, const double*
   lbo_status st = fx::tables(p, &tb);
   const int part = fx::part_size(p, B);
   if (st == LBO_OK)
-    st = fx::ensure(ws, ws_bytes, fx::q_workspace_bytes(p->N, part, p->J, rule.M, rule.omega3 != nullptr));
+    st = fx::ensure(ws, ws_bytes, fx::q_workspace_bytes(p->N, part, p->J, rule));
   const size_t n3 = (size_t)p->N * p->N * p->N;
   p->last_launches = 0;
   for (int b0 = 0; b0 < B && st == LBO_OK; b0 += part)

@@ -24,39 +24,46 @@ constexpr size_t H = (size_t)N * NC, n3 = (size_t)N * N * N;
 constexpr int ACC_WARPS = 8, PPC = PlanesPPC<N>::v, CPPC = CombinePPC<N>::v;
 
 // How a call is cut: G instances at a time whose J plane spectra PW stay below
-// 512 MB; of their (instance, node) pairs as many per launch, and of a pair's M
-// hemisphere nodes as many, as 1 GB of Z holds.
+// 512 MB; of a pair's hemisphere nodes as many classes per launch as keep their
+// Z and the table of e_2 e_3 below 1 GB each, and of the (instance, radial node)
+// pairs as many as 1 GB of Z holds.
 struct Cut {
-  int G, mc, pairs;
-  Cut(int B, int J, int M) {
-    const size_t z = sizeof(ci64) * n3;
-    G = (int)std::min<size_t>(B, std::max<size_t>(1, ((size_t)512 << 20) / (sizeof(ci64) * H * J)));
-    mc = (int)std::min<size_t>(M, std::max<size_t>(1, ((size_t)1 << 30) / z));
-    pairs = (int)std::min<size_t>((size_t)G * J, std::max<size_t>(1, ((size_t)1 << 30) / (z * mc)));
+  int G, classes, nodes, pairs;  // nodes: the most of a launch
+  Cut(int B, int J, const QuadRule& r) {
+    const size_t z = 2 * sizeof(ci64) * H, gb = (size_t)1 << 30;
+    G = (int)std::min<size_t>(B, std::max<size_t>(1, (gb / 2) / (sizeof(ci64) * H * J)));
+    int wide = 1;
+    for (int c = 0; c < r.classes; ++c) wide = std::max(wide, r.class_begin[c + 1] - r.class_begin[c]);
+    classes = (int)std::min<size_t>(r.classes, std::max<size_t>(1, std::min(gb / z, gb / (sizeof(ci64) * NC * J * wide))));
+    nodes = std::min(r.M, classes * wide);
+    const size_t all = (size_t)G * J, most = std::min<size_t>(all, std::max<size_t>(1, gb / (z * classes)));
+    const size_t launches = (all + most - 1) / most;
+    pairs = (int)((all + launches - 1) / launches);
   }
 };
 
 struct Buffers {
-  ci64 *R, *F, *PW, *Z, *tab;
+  ci64 *R, *F, *PW, *Z, *tab1, *tab;
   i64 *accG, *om3;
   double *BPh, *BP;
   float* rm;
   int *eR, *EF, *EPh, *EC, *bad, *EP, *accE;
   size_t bytes;
-  Buffers(void* base, size_t B, size_t J, size_t M, const Cut& c, bool position) {
+  Buffers(void* base, size_t B, size_t J, const QuadRule& r, const Cut& c) {
     unsigned char* p = (unsigned char*)base;
     auto take = [&](auto*& ptr, size_t count) {
       ptr = (std::remove_reference_t<decltype(ptr)>)p;
       p += (count * sizeof(*ptr) + 255) / 256 * 256;
     };
-    const bool rest = (size_t)c.mc < M;
+    const bool rest = c.classes < r.classes;
     take(R, B * H);
     take(F, 2 * B * H);
     take(PW, c.G * J * H);
-    take(Z, (size_t)c.pairs * c.mc * n3);
-    take(tab, J * M * 3 * N);
+    take(Z, (size_t)c.pairs * c.classes * 2 * H);
+    take(tab1, J * c.classes * N);
+    take(tab, J * c.nodes * NC);
     take(accG, rest ? c.pairs * n3 : 0);
-    take(om3, position ? H : 0);
+    take(om3, r.omega3 ? H : 0);
     take(BPh, B * N);
     take(BP, c.G * J * N);
     take(rm, B * BANDS * NC);
@@ -66,7 +73,7 @@ struct Buffers {
     take(EC, 2 * B * NC);
     take(bad, B);
     take(EP, c.G * J * N);
-    take(accE, rest ? (size_t)c.pairs * N : 0);
+    take(accE, rest ? (size_t)c.pairs * N * N : 0);
     bytes = (size_t)(p - (unsigned char*)base);
   }
 };
@@ -76,16 +83,16 @@ void smem_of(K kernel, size_t bytes) { raise_smem_limit((const void*)kernel, byt
 
 }  // namespace
 
-size_t LBO_CAT(q_workspace_bytes_, LBO_FX_N)(int B, int J, int M, bool position) {
-  return Buffers(nullptr, B, J, M, Cut(B, J, M), position).bytes;
+size_t LBO_CAT(q_workspace_bytes_, LBO_FX_N)(int B, int J, const QuadRule& rule) {
+  return Buffers(nullptr, B, J, rule, Cut(B, J, rule)).bytes;
 }
 
 lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const QuadRule& rule, const double* f, double* out,
                                        int B, void* ws) {
   cudaStream_t s = p->stream;
   const int J = p->J, M = rule.M;
-  const Cut cut(B, J, M);
-  const Buffers w(ws, B, J, M, cut, rule.omega3 != nullptr);
+  const Cut cut(B, J, rule);
+  const Buffers w(ws, B, J, rule, cut);
   cudaError_t e = cudaMemsetAsync(w.bad, 0, sizeof(int) * B, s);
   if (e != cudaSuccess) return cuda_fail(e, "fixed-point flags");
   const double pi = 3.141592653589793238462643383279502884;
@@ -96,9 +103,14 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   const double top = std::frexp(std::sqrt(rule.wmax * c0), &ke);  // top 2^ke, top in [0.5, 1)
   (void)top;
   const double c = std::scalbn(c0, -2 * ke);
-  LBO_LAUNCH(p, "q_fx_phase_table", s, k_q_phase_table<N>, J * M, 3 * N, 0, rule.gj, rule.sig, rule.wm, M, pi, 2.0 * p->L,
-             c, w.tab);
-  int launches = 5;
+  int launches = 4;
+  auto phases = [&](int c0, int c1) {
+    const int m0 = rule.class_begin[c0];
+    LBO_LAUNCH(p, "q_fx_phase_table", s, k_q_phase_table<N>, dim3(rule.class_begin[c1] - m0, J), 256, 0, rule.gj, rule.sig,
+               rule.wm, rule.node + m0, c0, c1 - c0, pi, 2.0 * p->L, c, w.tab1, w.tab);
+    launches += 1;
+  };
+  if (cut.classes == rule.classes) phases(0, rule.classes);
   const i64* omega = tb.omega;
   int omega_exp = tb.omega_exp;
   if (rule.omega3) {
@@ -116,21 +128,22 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   LBO_LAUNCH(p, "q_fx_rescale", s, k_q_rescale<N>, dim3((NC + 63) / 64, B), 64, 0, w.R, w.eR, w.rm, w.EF);
   smem_of(k_q_plane<N>, GeoQ<N>::BYTES);
   smem_of(k_axis1_acc<N, ACC_WARPS>, acc_smem<N, ACC_WARPS>(256));
-  // head room of the sum over m: products below 2^60
+  // head room of the sum over m: products of at most 2^60, a sum of at most 2^62
   int guard = 0;
-  while ((2 << guard) < M) ++guard;
+  while ((4 << guard) < M) ++guard;
   for (int b0 = 0; b0 < B; b0 += cut.G) {
     const int n = std::min(cut.G, B - b0);
     const ci64* R = w.R + b0 * H;
     for (int q0 = 0; q0 < n * J; q0 += cut.pairs) {
       const int np = std::min(cut.pairs, n * J - q0);
-      for (int m0 = 0; m0 < M; m0 += cut.mc) {
-        const int mc = std::min(cut.mc, M - m0);
-        LBO_LAUNCH(p, "q_fx_axis1_phase", s, k_q_axis1<N>, dim3((NC * T + 31) / 32, mc, np), 32, 0, R, w.tab, J, M, m0, q0,
+      for (int c0 = 0; c0 < rule.classes; c0 += cut.classes) {
+        const int c1 = std::min(c0 + cut.classes, rule.classes), m0 = rule.class_begin[c0], m1 = rule.class_begin[c1];
+        if (cut.classes < rule.classes) phases(c0, c1);
+        LBO_LAUNCH(p, "q_fx_axis1_phase", s, k_q_axis1<N>, dim3((NC * T + 31) / 32, c1 - c0, np), 32, 0, R, w.tab1, J, q0,
                    w.Z);
         LBO_LAUNCH(p, "q_fx_plane_prod", s, k_q_plane<N>, dim3(N / GeoQ<N>::PPC, np), GeoQ<N>::THREADS, GeoQ<N>::BYTES,
-                   w.Z, w.EF + b0, J, mc, q0, m0 == 0 ? 1 : 0, m0 + mc == M ? 1 : 0, guard, ke, w.accG, w.accE, w.PW, w.EP,
-                   w.BP);
+                   w.Z, w.tab, rule.node + m0, c0, c1 - c0, w.EF + b0, J, m1 - m0, q0, c0 == 0 ? 1 : 0,
+                   c1 == rule.classes ? 1 : 0, guard, ke, w.accG, w.accE, w.PW, w.EP, w.BP);
         launches += 2;
       }
     }

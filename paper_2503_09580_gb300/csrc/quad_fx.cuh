@@ -3,13 +3,18 @@
 // accumulation and combination kernels of L[g] (lin_fx.cuh).
 //
 // For radial node j and hemisphere node m the two translated fields T+ =
-// InvFFT(F E), T- = InvFFT(F conj E) are real, so one complex field Z = T+ + i T-
-// carries both through the planes: no packing of columns or rows, and the
-// product T+ T- is the product of a value's two parts.
+// InvFFT(F E), T- = InvFFT(F conj E), E = e_1 e_2 e_3, are real, so one complex
+// field Z = T+ + i T- carries both through the planes: no packing of columns or
+// rows, and the product T+ T- is the product of a value's two parts.  Since
+// E + i conj(E) = (1 + i) (Re E + Im E), Z = (1 + i) InvFFT(F (Re E + Im E)), and
+// with e_1 = c1 + i s1, e_2 e_3 = c + i s the multiplier is
+// c (c1 + s1) + s (c1 - s1): axis 1 only sees e_1, once for all nodes that share
+// |sigma_1|, four nodes of a ring as a rule (sigma and -sigma exchange T+ and
+// T-, so sigma_1 < 0 is taken as -sigma).
 //
-//   k_q_phase_table  the per-axis phase factors of every (j, m)
+//   k_q_phase_table  the phase factors of every radial node and hemisphere node
 //   k_q_rescale      F to one exponent per instance
-//   k_q_axis1        the axis-1 transform of Z for every m of a chunk
+//   k_q_axis1        the axis-1 transforms of Z for every class of nodes of a launch
 //   k_q_plane        axes 2 and 3 of Z, sum_m w_m T+ T- on chip, and the
 //                    forward transforms of axes 3 and 2 of the sum
 #pragma once
@@ -25,27 +30,53 @@ struct GeoQ {
   static constexpr bool WARP = TPP == 16 || TPP == 32;
   static constexpr int PPC = WARP ? 32 / TPP * 2 : (TPP == 24 ? 4 : 1);  // planes per block
   static constexpr int THREADS = TPP * PPC;
+  static constexpr int BLOCKS = Geo<N>::V == 16 ? 384 / THREADS : 1;  // per SM: 12 warps of 168 registers
   static constexpr int RS = T == 2 ? N + 2 : N + 1;  // row stride of the exchange buffer (Geo::RS)
   static constexpr size_t BYTES = (size_t)PPC * (sizeof(ci64) * N * RS + sizeof(i64) * N * N);
 };
 
-// tab[((j M + m) 3 + d) N + k] = exp(i alpha_d centred(k)) as two packed
-// multipliers (1 = 2^62), alpha_d = pi g_j sigma_(m,d) / (2 L), at the Nyquist
-// index cos(alpha_d N / 2), the average of the two images.  Axis 1 carries
-// s_m = sqrt(w_m c): T+ T- then carries w_m and the constant c.
-// grid = J M, block = 3 N.
+// Phase factors of radial node j and the nodes (-sigma where sigma_1 < 0) of a
+// launch, as packed multipliers.  e_d(k) = exp(i alpha_d centred(k)), alpha_d = pi g_j
+// sigma_(m,d) / (2 L), at the Nyquist index cos(alpha_d N / 2), the average of
+// the two images.  With e_1 = c + i s of a class, axis 1 takes
+//   tab1[(j classes + class) N + k1] = ((c + s) s_m, (c - s) s_m), 1 = 2^61,
+// where s_m = sqrt(w_m a): T+ T- then carries w_m and the constant a; the planes
+//   tab[(j nodes + node) NC + (k2, k3)] = e_2(k2) e_3(k3), 1 = 2^62.
+// grid = (nodes, J), block = 256.
 template <int N>
-__global__ void __launch_bounds__(3 * N) k_q_phase_table(const double* __restrict__ gj, const double* __restrict__ sig,
-                                                         const double* __restrict__ wm, int M, double pi, double two_l,
-                                                         double c, ci64* __restrict__ tab) {
-  const int j = blockIdx.x / M, m = blockIdx.x % M, d = threadIdx.x / N, k = threadIdx.x % N;
-  const double al = (pi * gj[j] / two_l) * sig[3 * m + d];
-  double s = 0.0, co;
-  if (k == N / 2) co = cos(al * (N / 2));
-  else sincos(al * (double)centred<N>(k), &s, &co);
-  const double f = d == 0 ? sqrt(wm[m] * c) : 1.0;
-  tab[(size_t)blockIdx.x * 3 * N + threadIdx.x] =
-      ci64{pack_mult(__double2ll_rn(co * f * 0x1p62)), pack_mult(__double2ll_rn(s * f * 0x1p62))};
+__global__ void __launch_bounds__(256) k_q_phase_table(const double* __restrict__ gj, const double* __restrict__ sig,
+                                                       const double* __restrict__ wm, const int4* __restrict__ node,
+                                                       int class0, int classes, double pi, double two_l, double a,
+                                                       ci64* __restrict__ tab1, ci64* __restrict__ tab) {
+  constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC;
+  __shared__ double2 e[2][N];
+  const int j = blockIdx.y;
+  const int4 nd = node[blockIdx.x];
+  const double f = (pi * gj[j] / two_l);
+  for (int t = threadIdx.x; t < 3 * N; t += 256) {
+    const int d = t / N, k = t % N;
+    if (d == 0 && !nd.w) continue;
+    const double sg = sig[3 * nd.x + d], al = f * (d == 0 ? fabs(sg) : nd.z ? -sg : sg);
+    double s = 0.0, co;
+    if (k == N / 2) co = cos(al * (N / 2));
+    else sincos(al * (double)centred<N>(k), &s, &co);
+    if (d == 0) {
+      const double sm = sqrt(wm[nd.x] * a) * 0x1p61;
+      tab1[((size_t)j * classes + nd.y - class0) * N + k] =
+          ci64{pack_mult(__double2ll_rn((co + s) * sm)), pack_mult(__double2ll_rn((co - s) * sm))};
+    } else {
+      e[d - 1][k] = double2{co, s};
+    }
+  }
+  __syncthreads();
+  ci64* out = tab + ((size_t)j * gridDim.x + blockIdx.x) * NC;
+  for (int t = threadIdx.x; t < NC; t += 256) {
+    const double2 u = e[0][t / HC], v = e[1][t % HC];
+    const i64 s = __double2ll_rn((u.x * v.y + u.y * v.x) * 0x1p62);
+    // the planes negate the words of s: its low one is not -2^31
+    out[t] = ci64{pack_mult(__double2ll_rn((u.x * v.x - u.y * v.y) * 0x1p62)),
+                  pack_mult((unsigned)(u64)s == 0x80000000u ? s + 1 : s)};
+  }
 }
 
 // The Eq. (2.16) loss multiplier (FP64, positions of fft.cuh along axes 1 and
@@ -93,112 +124,76 @@ __global__ void __launch_bounds__(64) k_q_rescale(ci64* __restrict__ R, const in
   }
 }
 
-__device__ __forceinline__ i64 raw_mult(i64 packed) {
-  const Mult m = unpack_mult(packed);
-  return ((i64)m.th << 32) + m.tl;
-}
-// (a, b) -> 4 a as a multiplier: products of two 2^62-scaled factors are 2^60-scaled
-__device__ __forceinline__ SignedMult times4_mult(i64 a) { return signed_mult((i64)((u64)a << 2)); }
-
-// Axis 1 of Z for the columns (k2, k3) of the half spectrum: Y+- =
-// InvFFT_1(F E), InvFFT_1(F conj E); Z(i1, k2, k3) = Y+ + i Y-, and at the
-// mirrored column Z(i1, -k2, -k3) = conj(Y+) + i conj(Y-).  One pass over F
-// forms both products, F conj E waits in shared memory.  E(-k1) shares E(k1)'s
-// four products.
-// Z: [bj][m][i1][k2][k3] of the launch; bj0: its first (instance, node) pair.
-// grid = (ceil(NC T / 32), mc, pairs), block = 32, shared memory V 32 words.
+// Axis 1 of Z for a class of hemisphere nodes, one thread per column (k2, k3)
+// of the half spectrum: S+- = InvFFT_1(F (c +- s)), stored as (1 + i) S+- in
+// Z[pair][class][i1][2][k2][k3]; real multipliers, two transforms for all nodes
+// of the class.  F (c - s) waits in shared memory.
+// Bound by the writes of Z (4.6 GB at N = 32, M = 32, 32 instances, 1.15 ms, 4.0
+// TB/s); one pass per node instead, with its own axis-1 products and 17 GB of Z,
+// took 7.3 ms.
+// tab1: [j][classes][N]; bj0: the launch's first (instance, radial node) pair.
+// grid = (ceil(NC T / 32), classes, pairs), block = 32, shared memory V 32 words.
 template <int N>
-__global__ void __launch_bounds__(32) k_q_axis1(const ci64* __restrict__ R, const ci64* __restrict__ tab, int J, int M,
-                                                int m0, int bj0, ci64* __restrict__ Z) {
-  constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, T = Geo<N>::T, V = Geo<N>::V;
+__global__ void __launch_bounds__(32) k_q_axis1(const ci64* __restrict__ R, const ci64* __restrict__ tab1, int J,
+                                                int bj0, ci64* __restrict__ Z) {
+  constexpr int NC = Geo<N>::NC, T = Geo<N>::T, V = Geo<N>::V;
   __shared__ ci64 S[V][32];
   const int lane = threadIdx.x, id = blockIdx.x * 32 + lane, h = T == 2 ? id & 1 : 0;
   const bool on = id / T < NC;
-  const int col = on ? id / T : NC - 1, k2 = col / HC, k3 = col % HC;
-  const int bj = bj0 + blockIdx.z, b = bj / J, j = bj % J, m = m0 + blockIdx.y;
-  const ci64* mf = tab + (size_t)(j * M + m) * 3 * N;
+  const int col = on ? id / T : NC - 1;
+  const int bj = bj0 + blockIdx.z, b = bj / J, j = bj % J;
+  const ci64* mf = tab1 + ((size_t)j * gridDim.y + blockIdx.y) * N;
   const ci64* src = R + (size_t)b * N * NC + col;
-  const ci64 e2 = mf[N + k2], e3 = mf[2 * N + k3];
-  const Mult e2x = unpack_mult(e2.x), e2y = unpack_mult(e2.y);
-  const ci64 c0 = cmul_mult(SignedMult{e2x, e2x.th >> 31}, SignedMult{e2y, e2y.th >> 31},
-                            ci64{raw_mult(e3.x), raw_mult(e3.y)});
-  const SignedMult cx = times4_mult(c0.x), cy = times4_mult(c0.y);
+  ci64* dst = Z + ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * N * 2 * NC + col;
   ci64 x[V];
-  // value i at k1 = k: F E in x, F conj(E) in S
-  auto product = [&](int i, int k, ci64 e) {
-    const ci64 f = src[(size_t)k * NC];
-    const SignedMult ex = times4_mult(e.x), ey = times4_mult(e.y);
-    const i64 ac = mul_signed(f.x, ex.m, ex.neg), bd = mul_signed(f.y, ey.m, ey.neg);
-    const i64 bc = mul_signed(f.y, ex.m, ex.neg), ad = mul_signed(f.x, ey.m, ey.neg);
-    x[i] = ci64{ac - bd, bc + ad};
-    S[i][lane] = ci64{ac + bd, bc - ad};
-  };
-  auto phase = [&](int k, ci64& e, ci64& em) {  // e1(k) c and conj(e1(k)) c
-    const ci64 a = mf[k];
-    const i64 ax = raw_mult(a.x), ay = raw_mult(a.y);
-    const i64 xx = mul_signed(ax, cx.m, cx.neg), yy = mul_signed(ay, cy.m, cy.neg);
-    const i64 xy = mul_signed(ax, cy.m, cy.neg), yx = mul_signed(ay, cx.m, cx.neg);
-    e = ci64{xx - yy, xy + yx};
-    em = ci64{xx + yy, xy - yx};
-  };
-  if constexpr (T == 1) {
 #pragma unroll
-    for (int k = 0; k <= N / 2; ++k) {
-      ci64 e, em;
-      phase(k, e, em);
-      product(k, k, e);
-      if (k > 0 && k < N / 2) product(N - k, N - k, em);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-      const int k = idx_parity<N>(i, h);
-      ci64 e, em;
-      phase(k, e, em);
-      product(i, k, e);
-    }
+  for (int i = 0; i < V; ++i) {
+    const int k = idx_parity<N>(i, h);
+    const ci64 f = src[(size_t)k * NC], e = mf[k];
+    const SignedMult p = signed_of(e.x), q = signed_of(e.y);
+    x[i] = ci64{mul_signed(f.x, p.m, p.neg), mul_signed(f.y, p.m, p.neg)};
+    S[i][lane] = ci64{mul_signed(f.x, q.m, q.neg), mul_signed(f.y, q.m, q.neg)};
   }
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
     dft_time<N, true>(x, h);
+    if (on) {
+#pragma unroll
+      for (int i = 0; i < V; ++i)  // (1 + i) x
+        dst[((size_t)idx_halves<N>(i, h) * 2 + pass) * NC] = ci64{x[i].x - x[i].y, x[i].x + x[i].y};
+    }
     if (pass == 0) {
 #pragma unroll
-      for (int i = 0; i < V; ++i) {
-        const ci64 v = S[i][lane];
-        S[i][lane] = x[i];
-        x[i] = v;
-      }
+      for (int i = 0; i < V; ++i) x[i] = S[i][lane];
     }
-  }
-  if (!on) return;
-  ci64* dst = Z + ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * N * N * N;
-  const size_t o = (size_t)k2 * N + k3, om = (size_t)((N - k2) % N) * N + (N - k3) % N;
-  const bool mirror = k3 > 0 && k3 < N / 2;
-#pragma unroll
-  for (int i = 0; i < V; ++i) {
-    const ci64 p = S[i][lane], q = x[i];
-    const size_t plane = (size_t)idx_halves<N>(i, h) * N * N;
-    dst[plane + o] = ci64{p.x - q.y, p.y + q.x};
-    if (mirror) dst[plane + om] = ci64{p.x + q.y, q.x - p.y};
   }
 }
 
-// One plane i1 of one (instance, node) pair: Z of every m of the launch through
-// the inverse axes 2 and 3, the sum over m of the products of its two parts
-// (kept in shared memory at the largest exponent met so far, `guard` bits
-// below a product's top), and after the last m the forward transforms of
+// One plane i1 of one (instance, radial node) pair: of every hemisphere node m of
+// the launch, Z from its class (k_q_axis1) and e_2 e_3, the inverse axes 2 and 3, the sum over m of the products of its two parts
+// (kept in shared memory, each row i2 at the largest exponent it met so far and
+// `guard` bits below a product's top), and after the last m the forward transforms of
 // axes 3 and 2 of the sum, two rows per pencil, into PW[bj][i1].  Between the
 // launches of a chunked m the sum rests in accG, accE.
+// node: the launch's mc nodes, of `classes` classes from class0 on.
+// Bound by instruction issue: 54 % of the slots at 12 warps per SM (168
+// registers; without the bound on registers, 8 warps, 14.8 ms), its integer pipe
+// 55 %; stalls are fixed latencies and instruction fetch.  N = 32, M = 32, 32
+// instances: 13.9 ms, where the kernel that read a ready Z per node took 10.1
+// and left 7.3 to axis 1.  The exponents of the sum belong to a row, not to the
+// plane: the largest T of a row needs a shuffle, that of a plane a barrier.
 // EF[b]: exponent of F; 2^ke: factor of the phase table; EP, BP as k_plane's.
 // grid = (N / PPC, pairs), block = GeoQ<N>::THREADS.
 template <int N>
-__global__ void __launch_bounds__(GeoQ<N>::THREADS) k_q_plane(const ci64* __restrict__ Z, const int* __restrict__ EF,
+__global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(const ci64* __restrict__ Z,
+                                                            const ci64* __restrict__ tab, const int4* __restrict__ node,
+                                                            int class0, int classes, const int* __restrict__ EF,
                                                             int J, int mc, int bj0, int first, int last, int guard, int ke,
                                                             i64* __restrict__ accG, int* __restrict__ accE,
                                                             ci64* __restrict__ PW, int* __restrict__ EP,
                                                             double* __restrict__ BP) {
   using G = GeoQ<N>;
-  constexpr int NC = Geo<N>::NC, T = Geo<N>::T, V = Geo<N>::V, TPP = G::TPP, RS = G::RS, FT = Geo<N>::TPP;
+  constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, T = Geo<N>::T, V = Geo<N>::V, TPP = G::TPP, RS = G::RS, FT = Geo<N>::TPP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned red[5 * G::PPC];
   const int pp = threadIdx.x / TPP, tp = threadIdx.x % TPP, h = T == 2 ? tp & 1 : 0, q = tp / T;
@@ -223,17 +218,18 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS) k_q_plane(const ci64* __rest
     }
   };
   if (threadIdx.x < 5 * G::PPC) red[threadIdx.x] = 0;
-  int EA = kZeroExp;  // exponent of the sum
+  int EA = kZeroExp;  // exponent of the pencil's sum
   if (first) {
 #pragma unroll
     for (int i = 0; i < V; ++i) acc[idx_halves<N>(i, h) * N + q] = 0;
   } else {
 #pragma unroll
     for (int i = 0; i < V; ++i) acc[idx_halves<N>(i, h) * N + q] = accG[pl * N * N + idx_halves<N>(i, h) * N + q];
-    EA = accE[pl];
+    EA = accE[pl * N + q];
   }
   __syncthreads();
-  const int E0 = EF[bj / J] + 2 + ke;  // products with the 2^62-scaled phases, 2^ke in axis 1's
+  // products with the 2^61-scaled axis-1 factors, which carry 2^ke, and with e_2 e_3
+  const int E0 = EF[bj / J] + 5 + ke;
   const PlaneThread t{pp, tp, h, q};
   const bool fwd = tp < FT;  // threads of the forward pencils
   ci64 x[V];
@@ -244,15 +240,38 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS) k_q_plane(const ci64* __rest
   for (int it = 0; it < passes; ++it) {
     const int kind = it >= 2 * mc ? 2 + (it - 2 * mc) : it & 1;
     if (kind == 0) {
-      const ci64* src = Z + (((size_t)blockIdx.y * mc + (it >> 1)) * N + i1) * N * N + q;
+      // Z(k2, q) = c Z1 + s Z2, e_2 e_3 = c + i s.  Beyond the half spectrum,
+      // from its mirrored entry: the parts of c Z2 - s Z1, exchanged.
+      const int4 nd = node[it >> 1];
+      const bool mir = q > N / 2;
+      const size_t o = (mir ? (size_t)N * HC + N - q : (size_t)q);
+      const int step = mir ? -HC : HC;
+      const ci64* z = Z + ((((size_t)blockIdx.y * classes + nd.y - class0) * N + i1) * 2) * NC;
+      const ci64 *z1 = z + (mir ? NC : 0) + o, *z2 = z + (mir ? 0 : NC) + o;
+      const ci64* ph = tab + ((size_t)(bj % J) * mc + (it >> 1)) * NC + o;
+      const int flip = mir ? -1 : 0;
 #pragma unroll
-      for (int i = 0; i < V; ++i) x[i] = src[(size_t)idx_parity<N>(i, h) * N];
+      for (int i = 0; i < V; ++i) {
+        const int k = idx_parity<N>(i, h), r = (mir && k == 0 ? N : k) * step;
+        const ci64 u = z1[r], v = z2[r], e = ph[r];
+        const Mult c = unpack_mult(e.x), sw = unpack_mult(e.y), sn = Mult{(sw.th ^ flip) - flip, (sw.tl ^ flip) - flip};
+        const i64 zx = mul_pair(u.x, c, v.x, sn), zy = mul_pair(u.y, c, v.y, sn);
+        x[i] = ci64{mir ? zy : zx, mir ? zx : zy};
+      }
       E = E0;
     } else if (kind == 1) {
 #pragma unroll
       for (int i = 0; i < V; ++i) x[i] = Bs[q * RS + idx_parity<N>(i, h)];
     } else if (kind == 2) {
-      // rows q and q + N/2 of the sum, parts exchanged
+      // the rows to one exponent; rows q and q + N/2 of the sum, parts exchanged
+      const int top = (int)group_max((unsigned)(EA - 2 * kZeroExp), 4) + 2 * kZeroExp, d = min(top - EA, 63);
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        i64& a = acc[idx_halves<N>(i, h) * N + q];
+        a = shift_right(a, d);
+      }
+      EA = top;
+      sync();
 #pragma unroll
       for (int i = 0; i < V; ++i) {
         const i64* a = acc + idx_halves<N>(i, h) * N;
@@ -270,19 +289,24 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS) k_q_plane(const ci64* __rest
     if (kind == 0) {
 #pragma unroll
       for (int i = 0; i < V; ++i) Bs[idx_halves<N>(i, h) * RS + q] = x[i];
-      if (!G::WARP && threadIdx.x < G::PPC) red[4 * G::PPC + threadIdx.x] = red[G::PPC + threadIdx.x] = 0;
+      if (!G::WARP && threadIdx.x < G::PPC) red[G::PPC + threadIdx.x] = 0;
       sync();
-    } else if (kind == 1) {
-      // T+ and T- to a top bit of 2^61, their product, and the sum over m
-      unsigned m = top_bits<V>(x);
-      m = group_max(m, 4);
       if (!G::WARP && threadIdx.x < G::PPC) red[threadIdx.x] = 0;
-      const int l = m ? __clz(m) - 1 : 0;
-      const int EPr = 2 * (E - l) + 64 + guard;
+    } else if (kind == 1) {
+      // T+ and T- of the pencil to at most 2^62, their product, and the sum over m
+      int m = 0;
+#pragma unroll
+      for (int i = 0; i < V; ++i) m = max(m, max(abs((int)(x[i].x >> 32)), abs((int)(x[i].y >> 32))));
+      if (T == 2) m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+      const int l = max(__clz(m) - 2, 0);
+      const int EPr = m ? 2 * (E - l) + 64 + guard : kZeroExp;
       if (EPr > EA) {  // the sum moves to the larger exponent
         const int d = min(EPr - EA, 63);
 #pragma unroll
-        for (int i = 0; i < V; ++i) acc[idx_halves<N>(i, h) * N + q] >>= d;
+        for (int i = 0; i < V; ++i) {
+          i64& a = acc[idx_halves<N>(i, h) * N + q];
+          a = shift_right(a, d);
+        }
         EA = EPr;
       }
       const int d = min(EA - EPr + guard, 62);
@@ -293,7 +317,6 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS) k_q_plane(const ci64* __rest
         const i64 p = mul_signed_rounded((i64)((u64)x[i].x << l), a.m, a.neg);
         acc[idx_halves<N>(i, h) * N + q] += (p + half) >> d;
       }
-      sync();
     } else if (kind == 2) {
       sync();
       if (fwd) store_rows<N>(x, t, Bs);
@@ -303,7 +326,7 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS) k_q_plane(const ci64* __rest
   if (!last) {
 #pragma unroll
     for (int i = 0; i < V; ++i) accG[pl * N * N + idx_halves<N>(i, h) * N + q] = acc[idx_halves<N>(i, h) * N + q];
-    if (tp == 0) accE[pl] = EA;
+    if (h == 0) accE[pl * N + q] = EA;
     return;
   }
   if (!fwd) return;

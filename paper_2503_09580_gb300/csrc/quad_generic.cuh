@@ -28,6 +28,7 @@ namespace lbo {
 struct QuadState {
   int p = 0;                   // hemisphere order of the cached rule
   std::vector<double> sig, wm;  // M x 3, M
+  std::vector<int> order, class_begin;  // nodes grouped by |sigma_1| and weight
   // loss multiplier of Eq. (2.16) per half-spectrum position, in the
   // transform precision of omq_prec, for hemisphere order omq_p
   void* d_omq = nullptr;

@@ -13,6 +13,7 @@
 // transforms + J forward transforms + 4.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "lin_fx.h"
@@ -39,6 +40,26 @@ void hemisphere_rule(int p, std::vector<double>& sig, std::vector<double>& wm) {
       sig.push_back(mu);
       wm.push_back(0.5 * w[a] / na);
     }
+  }
+}
+
+// The nodes ordered by classes of equal |sigma_1| and weight: e^(i alpha_1 k_1)
+// of a class is one pair of factors (quad_fx.cuh).  The azimuths of a ring share
+// |cos| in fours (in twos at +-90 degrees), up to the rounding of cos.
+void node_classes(const std::vector<double>& sig, const std::vector<double>& wm, std::vector<int>& order,
+                  std::vector<int>& begin) {
+  const int M = (int)wm.size();
+  std::vector<char> taken(M, 0);
+  order.clear();
+  begin.assign(1, 0);
+  for (int a = 0; a < M; ++a) {
+    if (taken[a]) continue;
+    for (int b = a; b < M; ++b)
+      if (!taken[b] && wm[b] == wm[a] && std::fabs(std::fabs(sig[3 * b]) - std::fabs(sig[3 * a])) < 1e-15) {
+        taken[b] = 1;
+        order.push_back(b);
+      }
+    begin.push_back((int)order.size());
   }
 }
 
@@ -172,6 +193,7 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
   }
   if (qs->p != p->hemi_p) {
     hemisphere_rule(p->hemi_p, qs->sig, qs->wm);
+    node_classes(qs->sig, qs->wm, qs->order, qs->class_begin);
     qs->p = p->hemi_p;
   }
   // the fused FP32 kernels take the radial loss multiplier only
@@ -208,6 +230,15 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
       std::vector<double> h(p->gj);
       h.insert(h.end(), qs->sig.begin(), qs->sig.end());
       h.insert(h.end(), qs->wm.begin(), qs->wm.end());
+      h.resize((h.size() + 1) / 2 * 2);  // the nodes by class, four ints each
+      for (size_t k = 0, c = 0; k < qs->order.size(); ++k) {
+        if ((int)k == qs->class_begin[c + 1]) ++c;
+        const int m = qs->order[k], first = (int)k == qs->class_begin[c];
+        const int nd[4] = {m, (int)c, qs->sig[3 * m] < 0.0, first};
+        double w[2];
+        std::memcpy(w, nd, sizeof(nd));
+        h.insert(h.end(), w, w + 2);
+      }
       e = cudaMalloc(&qs->d_gsw, sizeof(double) * h.size());
       if (e == cudaSuccess) e = cudaMemcpy(qs->d_gsw, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice);
       if (e != cudaSuccess) return cuda_fail(e, "quadrature nodes upload");
@@ -234,7 +265,9 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
     double bound = 0.0;
     for (int j = 0; j < p->J; ++j) bound += std::fabs(p->wj[j] * p->Bj[j]);
     bound *= 16.0 * 3.141592653589793 * 3.141592653589793 / ((double)p->N * p->N * p->N);
-    const fx::QuadRule rule{qs->d_gsw, dsig, dsig + 3 * M, M, *std::max_element(qs->wm.begin(), qs->wm.end()),
+    const int4* node = (const int4*)(qs->d_gsw + (p->J + 4 * M + 1) / 2 * 2);
+    const fx::QuadRule rule{qs->d_gsw, dsig, dsig + 3 * M, M, node, qs->class_begin.data(),
+                            (int)qs->class_begin.size() - 1, *std::max_element(qs->wm.begin(), qs->wm.end()),
                             (const double*)omq, bound};
     return run_quadratic_fx(p, rule, f, out, B, &qs->ws, &qs->ws_bytes);
   }

@@ -93,7 +93,28 @@ static void product(const char* name, bool sign, int ybits, F f) {
   std::printf("%s %.3f %.4f\n", name, worst, bias);
 }
 
+// mul_pair(): random directions (t, w) of norm 2^62 and below
+static void pair() {
+  double worst = 0, bias = 0;
+  const int n = 200000;
+  for (int tr = 0; tr < n; ++tr) {
+    i64 y = (i64)(rng() >> 4), z = (i64)(rng() >> 4);
+    if (rng() & 1) y = -y;
+    if (rng() & 1) z = -z;
+    const long double a = (rng() >> 11) * 0x1p-53L * 2 * 3.14159265358979323846L;
+    const i64 t = (i64)(cosl(a) * 0x1p62L), w = (i64)(sinl(a) * 0x1p62L) >> (tr % 3 == 0 ? rng() % 50 : 0);
+    if (tr % 1000 == 0) y = z = 0;
+    const __int128 p = (__int128)y * t + (__int128)z * w;
+    const double e = (double)(mul_pair(y, unpack_mult(pack_mult(t)), z, unpack_mult(pack_mult(w))) - (i64)(p >> 64)) -
+                     (double)(unsigned long long)p / 18446744073709551616.0;
+    worst = fmax(worst, fabs(e));
+    bias += e / n;
+  }
+  std::printf("mul_pair %.3f %.4f\n", worst, bias);
+}
+
 int main() {
+  pair();
   product("mul", false, 60, [](i64 y, Mult m) { return mul(y, m); });
   product("mul_signed", true, 62, [](i64 y, Mult m) { return mul_signed(y, m, m.th >> 31); });
   product("mul_signed_rounded", true, 62, [](i64 y, Mult m) { return mul_signed_rounded(y, m, m.th >> 31); });

@@ -83,7 +83,7 @@ def test_scale_and_degenerate_inputs():
 
 @pytest.mark.parametrize("n,batch,J,p,kw", [(16, 5, 16, 1, {}), (16, 1, 3, 5, {"q_sinc_quadrature": 1}), (24, 3, 24, 2, {}),
                                             (32, 3, 32, 4, {}), (32, 2, 5, 2, {"q_sinc_quadrature": 1}), (48, 2, 4, 3, {}),
-                                            (64, 1, 12, 4, {})])
+                                            (64, 1, 12, 4, {}), (64, 1, 64, 16, {})])  # the last in two cuts of its nodes
 def test_quadratic_matches_the_fp64_kernels(n, batch, J, p, kw):
     L = 8.0
     _, g = workloads.batched_instances(n, L, batch=batch, seed=90 + n, noise=0.0)
@@ -100,3 +100,37 @@ def test_quadratic_matches_the_fp64_kernels(n, batch, J, p, kw):
     if batch > 1:
         assert np.all(c[0] == 0)
         assert all(np.array_equal(c[i], a[i]) for i in range(1, batch - 1))
+
+
+@pytest.mark.parametrize("n", [16, 24, 32, 48, 64])
+def test_pairs_of_fp32_stay_reachable(n):
+    """FP32X2 runs in fixed point by default, bit for bit as FP64 does;
+    kernel = 1 still selects the pairs of FP32, within their 2^-48 bound."""
+    L = 8.0
+    params, g = workloads.batched_instances(n, L, batch=2, seed=110 + n, noise=1e-3)
+    a = apply(lbo.Plan(n, L, 0.5, n), params, g)
+    assert np.array_equal(a, apply(lbo.Plan(n, L, 0.5, n, precision="fp32x2"), params, g))
+    b = apply(lbo.Plan(n, L, 0.5, n, precision="fp32x2", kernel=1), params, g)
+    assert not np.array_equal(a, b)
+    tol = 4 * (2.0 ** -48 + U64) * np.maximum(ratio_rms(params, g, n, L), 64.0)
+    for i in range(2):
+        assert np.abs(a[i] - b[i]).max() <= tol[i] * np.abs(b[i]).max()
+
+
+@pytest.mark.parametrize("n,precision", [(16, "fp64"), (32, "fp32x2")])
+def test_cut_off_changed_after_the_maxwellian_cache(n, precision):
+    """The cached tables that depend on the cut-off level are made again when
+    it changes: cached and plain applications stay equal bit for bit."""
+    L = 8.0
+    params, g = workloads.batched_instances(n, L, batch=3, seed=120, noise=1e-3)
+    tp, tg = torch.from_numpy(params).to(DEV), torch.from_numpy(g).to(DEV)
+    plan, plain = (lbo.Plan(n, L, 0.5, n, precision=precision) for _ in range(2))
+    plan.cache_maxwellians(tp)
+    for eps in (1e-9, 1e-5, 1e-9):
+        plan.set("eps", eps)
+        plain.set("eps", eps)
+        a, b = torch.empty_like(tg), torch.empty_like(tg)
+        plan.apply_linearized(tp, tg, a)
+        plain.apply_linearized(tp, tg, b)
+        plan.sync(), plain.sync()
+        assert torch.equal(a, b)

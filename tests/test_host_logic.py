@@ -82,6 +82,7 @@ def test_fixed_point_arithmetic_against_long_double(tmp_path):
     res = {r[0]: (float(r[1]), float(r[2])) for r in (line.split() for line in out.strip().splitlines())}
     assert res["mul"][0] < 1.5 and res["mul_signed"][0] < 1.5 and res["mul_signed_rounded"][0] < 1.0
     assert abs(res["mul_signed_rounded"][1]) < 0.01
+    assert res["mul_pair"][0] < 2 * 1.5  # the sum of two products
     for n in (16, 24, 32):
         for d in "fi":
             err, bias = res["dft%d%s" % (n, d)]
