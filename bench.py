@@ -5,8 +5,9 @@ background Maxwellians rho ~ U[0.5,2], u_i ~ U[-0.5,0.5], theta ~ U[0.5,2],
 g = M * (quartic polynomial, N(0,1) coefficients) + 1e-3 N(0,1) grid noise.
 
 One step = one lbo_apply_linearized call over the whole batch (every kernel
-of the path).  The headline value is the plain FP64 path (the paper's
-arithmetic); the FP32 form, the VHS exponents 0.5 / 0.74 / 1.0 and the
+of the path).  The headline value is the FP64 path (FP64 data and
+Maxwellians, transforms in 64-bit fixed point that err no more than FP64
+ones); the same path with FP64 transforms throughout, the FP32 form, the VHS exponents 0.5 / 0.74 / 1.0 and the
 solver and N = 64 workloads are reported beside it, each precision form
 with its measured error against the oracle and its stated bound.  The ALU
 peaks of the roofline fractions are measured in the run
@@ -51,17 +52,20 @@ UNIT_ROUNDOFF = {"fp64": U64, "fp32": U32, "fp32x2": 2.0 ** -48, "fp64x2": 2.0 *
 BOUND_FACTOR = 4.0
 HBM_FALLBACK_GBS = 6800.0
 # Kernels bound by memory traffic, not by their arithmetic (rated in GB/s).
-HBM_KERNELS = ("combine", "conservation_fix", "f32_head", "f32_tail", "tc_combine", "mh_table")
+HBM_KERNELS = ("combine", "conservation_fix", "f32_head", "f32_tail", "tc_combine", "mh_table", "fx_mh_table")
+# Fixed-point transforms (fx64.cuh) run on the integer pipe.  Their peak: a
+# 32-point complex transform held in registers, nothing else running, takes 22
+# SM clocks per transform (measured on a GB300, all warps busy): 2.5 * 2 * 32 *
+# log2(32) = 800 conventional flops, 36.4 per SM and clock.
+FX_FLOPS_PER_SM_CLOCK = 800.0 / 22.0
 # DRAM bytes (read + write) per launch of a dominant kernel at the benchmark
 # workload from one ncu capture, with the sha256 (first 16 hex digits) of the
 # source files it was built from; reported as null once those sources change.
 KERNEL_SOURCES = {
-    "plane_inv_mh_fwd": ("lin_reg64.cuh", "fft_reg.cuh", "fft.cuh", "twiddles_hi.h"),
+    "fx_plane_inv_mh_fwd": ("lin_fx.cuh", "fx64.cuh", "fx_constants.h"),
     "f32_gain": ("lin_fused32.cu", "fused32.cuh", "tmem.cuh"),
 }
 NCU_TRAFFIC = {
-    # one capture of k_plane_mh_r64<8> at the benchmark workload: 138.75 MB read + 26.02 MB written
-    ("plane_inv_mh_fwd", 32, "fp64"): (164766208, "c353d0056c0cbfeb"),
 }
 
 
@@ -134,10 +138,24 @@ KERNEL_POINTWISE = {  # flops per grid point per instance
 #   back);  tail: the inverse of L^+ (1).
 FUSED_TRANSFORMS = {"f32_head": lambda J: 1, "f32_gain": lambda J: 2 * J + 4, "f32_tail": lambda J: 1}
 FUSED_POINTWISE = {"f32_gain": lambda J: 10 * J}
+# Fixed-point kernels: (axis passes, flops per grid point, octants) per
+# instance of one application; a launch covers all radial nodes of a group of
+# instances.  Head: the forward axes of r and g, axis 1 of r^, and both ways of
+# g^ omega; M^ comes from products of 1-D transforms and goes back alone.
+FX_KERNELS = {
+    "fx_plane_fwd": lambda J: (4, 0, 0), "fx_axis1_head": lambda J: (4, 4, 0), "fx_uhat": lambda J: (0, 0, J),
+    "fx_axis1_uhat_inv": lambda J: (J, 3 * J, 0), "fx_plane_inv_mh_fwd": lambda J: (4 * J, 2 * J, 0),
+    "fx_axis1_fwd_acc": lambda J: (J + 1, 4 * J, 0), "fx_combine": lambda J: (6, 5, 0),
+}
+# tables and bounds, no transform and little memory: not rated
+FX_SETUP = ("fx_instance", "fx_unit_scale")
 
 
 def kernel_flops_per_instance(name, n, J=None):
     J = n if J is None else J
+    if name in FX_KERNELS:
+        passes, point, octants = FX_KERNELS[name](J)
+        return passes * transform_axis_flops(n) + point * n ** 3 + octants * DCT_KERNELS["uhat_octant"](n, J)
     extra = DCT_KERNELS[name](n, J) if name in DCT_KERNELS else 0
     if name == "f32_uhat":
         return extra
@@ -163,7 +181,7 @@ def kernel_bytes_per_instance(name, n, real_bytes, groups=1):
         return groups * 8 * h + 4 * n3 + 8 * n3
     if name == "tc_combine":   # L+, u (FP64), w (FP32), g in; out
         return 8 * n3 * 4 + 4 * n3
-    if name == "mh_table":     # M^h / 2 of the register plane kernel out (FP64)
+    if name in ("mh_table", "fx_mh_table"):     # the M^h table out (64 bits a point)
         return 8 * n3
     return 0
 
@@ -179,7 +197,20 @@ def tensor_peak():
         return 1700.0, "fallback (sustained bf16 GEMM of an earlier GB300 measurement)"
 
 
-def kernel_rooflines(prof, n, batch, peak_tflops, hbm_gbs, real_bytes, groups=1):
+def fx_peak_tflops(peaks):
+    """Rate of the fixed-point register transforms on the integer pipe."""
+    return FX_FLOPS_PER_SM_CLOCK * peaks["sm_count"] * peaks["sm_mhz"] * 1e6 / 1e12
+
+
+def instances_per_launch(prof, name, batch):
+    """The fixed-point gain loop runs a batch in groups of instances; every
+    application has one fx_combine launch (at the batches timed here)."""
+    if not name.startswith("fx_") or "fx_combine" not in prof:
+        return batch
+    return batch * prof["fx_combine"][0] / max(prof[name][0], 1)
+
+
+def kernel_rooflines(prof, n, batch, peak_tflops, hbm_gbs, real_bytes, groups=1, fx_peak=None):
     """Per kernel: average launch time (live CUDA events) and its own bound:
     algorithmic flops against the measured ALU peak, or compulsory bytes
     against the measured HBM bandwidth for the memory-bound kernels.  The
@@ -187,7 +218,9 @@ def kernel_rooflines(prof, n, batch, peak_tflops, hbm_gbs, real_bytes, groups=1)
     (2n x 2n) real DFT matrix per pencil of n complex values: 6 (2n)^2 per
     pencil, n^2 pencils per instance) against the measured sustained tensor
     peak, and their bytes (read and write of a complex FP32 field, plus the
-    FP64 input or output of the first and last passes) against HBM."""
+    FP64 input or output of the first and last passes) against HBM.  The
+    fixed-point kernels (fx_*): algorithmic flops against fx_peak, the rate of
+    their register transforms alone on the integer pipe."""
     out = {}
     tpk, _ = tensor_peak()
     for name, (cnt, tot) in sorted(prof.items()):
@@ -202,14 +235,23 @@ def kernel_rooflines(prof, n, batch, peak_tflops, hbm_gbs, real_bytes, groups=1)
                         "frac_of_hbm": gbs / hbm_gbs})
             out[name] = rec
             continue
+        if name in FX_SETUP:
+            rec["bound"] = "latency"
+            out[name] = rec
+            continue
+        insts = instances_per_launch(prof, name, batch)
         if name in HBM_KERNELS:
-            by = kernel_bytes_per_instance(name, n, real_bytes, groups) * batch
+            by = kernel_bytes_per_instance(name, n, real_bytes, groups) * insts
             ach = by / (per * 1e-3) / 1e9 if per > 0 else 0.0
             rec.update({"bound": "hbm", "achieved_gbs": ach, "frac": ach / hbm_gbs})
         else:
-            fl = kernel_flops_per_instance(name, n) * batch
+            fl = kernel_flops_per_instance(name, n) * insts
             ach = fl / (per * 1e-3) / 1e12 if per > 0 else 0.0
-            rec.update({"bound": "alu", "achieved_tflops": ach, "frac": ach / peak_tflops})
+            fixed = name in FX_KERNELS and fx_peak
+            rec.update({"bound": "integer alu" if fixed else "alu", "achieved_tflops": ach,
+                        "frac": ach / (fx_peak if fixed else peak_tflops)})
+            if fixed:
+                rec["frac_of_fp64_peak"] = ach / peak_tflops
         out[name] = rec
     return out
 
@@ -460,11 +502,16 @@ def dominant_roofline(prof, precision, peaks, hbm, hbm_src, groups=1):
         ach = kernel_bytes_per_instance(name, N_GRID, real_bytes, groups) * BATCH / (per * 1e-3) / 1e9
         rf = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "peak_source": hbm_src}
     else:
-        ach = kernel_flops_per_instance(name, N_GRID) * BATCH / (per * 1e-3) / 1e12
+        ach = kernel_flops_per_instance(name, N_GRID) * instances_per_launch(prof, name, BATCH) / (per * 1e-3) / 1e12
         pk = peaks["fp64_tflops"] if precision == "fp64" else peaks["fp32_tflops"]
         rf = {"bound": "alu", "achieved": ach, "peak": pk, "unit": "TFLOP/s",
               "peak_source": "measured in this run (lbo_measure_alu_peaks: dense %s chains, %d SMs at %.0f MHz)"
                              % ("DFMA" if precision == "fp64" else "FFMA", peaks["sm_count"], peaks["sm_mhz"])}
+        if name in FX_KERNELS:
+            rf.update({"bound": "integer alu", "peak": fx_peak_tflops(peaks), "frac_of_fp64_peak": ach / peaks["fp64_tflops"],
+                       "peak_source": "64-bit fixed-point 32-point transforms in registers, %.1f conventional flops per "
+                                      "SM and clock measured, %d SMs at %.0f MHz of this run"
+                                      % (FX_FLOPS_PER_SM_CLOCK, peaks["sm_count"], peaks["sm_mhz"])})
     rf.update({"frac": rf["achieved"] / rf["peak"], "traffic": ncu_traffic(name, N_GRID, precision),
                "kernel": name, "kernel_share": share, "kernel_ms_per_launch": per,
                "apply_flops_per_instance": apply_flops_per_instance(N_GRID, N_GRID)})
@@ -488,12 +535,13 @@ def variant_leg(precision, tp, tg, tpc, tgc, stream, steps, peaks, hbm, ref, ref
     ms, prof, launches = time_steps(plan, tp, tg, out, steps, stream, True)
     unit = UNIT_ROUNDOFF[precision]
     real_bytes = 8 if precision in ("fp64", "fp32x2") else 4
-    # the pairs of FP32 run on the FP32 pipe: their algorithmic (FP64-class)
-    # flop rate is rated against the FFMA peak, and also shown against the
-    # DFMA peak of the FP64 form they replace
-    peak = peaks["fp64_tflops"] if precision == "fp64" else peaks["fp32_tflops"]
-    kr = kernel_rooflines(prof, N_GRID, BATCH, peak, hbm, real_bytes, groups or 1)
-    if precision == "fp32x2":
+    # the pairs of FP32 (kernel = 1) run on the FP32 pipe: their algorithmic
+    # (FP64-class) flop rate is rated against the FFMA peak, and also shown
+    # against the DFMA peak of the FP64 form they replace
+    pairs = precision == "fp32x2" and kernel != 0
+    peak = peaks["fp64_tflops"] if precision in ("fp64", "fp32x2") and not pairs else peaks["fp32_tflops"]
+    kr = kernel_rooflines(prof, N_GRID, BATCH, peak, hbm, real_bytes, groups or 1, fx_peak_tflops(peaks))
+    if pairs:
         for rec in kr.values():
             if "achieved_tflops" in rec:
                 rec["frac_of_fp64_peak"] = rec["achieved_tflops"] / peaks["fp64_tflops"]
@@ -989,7 +1037,8 @@ def quadratic_leg(precision, peaks, batch=128, steps=3, n=32, L=8.0, p=4, kernel
     evaluations/s and the rooflines of its two per-(j, m) kernels (their
     algorithmic work per radial and hemisphere node and instance:
     q_axis1_phase 2 axis passes + the phase products, q_plane_inv_prod 4 axis
-    passes + the product)."""
+    passes + the product; the fixed-point q_fx_plane_prod also takes the sum
+    over m through two forward passes)."""
     import torch
     from paper_2503_09580_gb300 import lbo, workloads
     _, g = workloads.batched_instances(n, L, batch=batch, seed=3, noise=0.0)
@@ -1016,6 +1065,8 @@ def quadratic_leg(precision, peaks, batch=128, steps=3, n=32, L=8.0, p=4, kernel
     peak = peaks["fp64_tflops"] if precision == "fp64" else peaks["fp32_tflops"]
     work = {"q_axis1_phase": 2 * transform_axis_flops(n) + 9 * n ** 3,
             "q_plane_inv_prod": 4 * transform_axis_flops(n) + 2 * n ** 3}
+    work["q_fx_axis1_phase"] = work["q_axis1_phase"]
+    work["q_fx_plane_prod"] = work["q_plane_inv_prod"] + 2 * transform_axis_flops(n) / M
     kr = {}
     for name, (cnt, tot) in sorted(prof.items()):
         per = tot / max(cnt, 1)
@@ -1023,7 +1074,7 @@ def quadratic_leg(precision, peaks, batch=128, steps=3, n=32, L=8.0, p=4, kernel
         if name in work and precision != "fp32":
             fl = work[name] * batch * (J * M / cnt)  # (j, m) pairs per launch
             rec.update({"bound": "alu", "achieved_tflops": fl / (per * 1e-3) / 1e12})
-            rec["frac"] = rec["achieved_tflops"] / peak
+            rec["frac"] = rec["achieved_tflops"] / (fx_peak_tflops(peaks) if name.startswith("q_fx_") else peak)
         kr[name] = rec
     return {"workload": "Q(f,f), N=32, M=32 hemisphere points, J=32, hard spheres, batch %d" % batch,
             "precision": precision, "kernel_set": {0: "fastest", 2: "shared-memory transforms"}.get(kernel, kernel),
@@ -1081,7 +1132,7 @@ def run_ours(args, world, rank, local):
         plan.set("moment_fix", 1)
     out = torch.empty_like(tg)
     # launch shape timed on this batch: radial-node groups per CTA of the
-    # fused FP32 kernel, or planes per CTA of the FP64 register plane kernel
+    # fused FP32 kernel, or planes per CTA of the FP64 plane kernel
     shape = plan.autotune(tp, tg, out) if prec in ("fp32", "fp64") and not args.no_autotune else 0
     jgroups = shape if prec == "fp32" else 0
     for _ in range(args.warmup):
@@ -1097,7 +1148,7 @@ def run_ours(args, world, rank, local):
     ms_max = max_over_ranks(ms, world)
     value = world * BATCH / (ms_max * 1e-3)
     real_bytes = 4 if prec == "fp32" else 8
-    peak = peaks["fp64_tflops"] if prec == "fp64" else peaks["fp32_tflops"]
+    peak = peaks["fp64_tflops"] if prec in ("fp64", "fp32x2") else peaks["fp32_tflops"]
 
     # end to end through the same C-ABI call with pinned host buffers
     hp = torch.from_numpy(params).pin_memory()
@@ -1112,6 +1163,8 @@ def run_ours(args, world, rank, local):
     cfg = workload_config(args.omega, prec)
     cfg.update({"eps": args.eps if args.eps is not None else 1e-9,
                 "jgroups": jgroups if jgroups else "n/a",
+                "transforms": "64-bit block fixed point on the integer pipe, FP64 in and out; error stated beside "
+                              "the value" if prec in ("fp64", "fp32x2") else "FP32",
                 "planes_per_cta": shape if prec == "fp64" and shape else "n/a",
                 "parallelism": "replicas (instances sharded, no collective)" if world > 1 else "single GPU",
                 "l2": "inputs 67 MB + outputs 67 MB + workspace per step > 129 MB L2"})
@@ -1121,7 +1174,8 @@ def run_ours(args, world, rank, local):
         "vs_baseline": None, "dtype": {"fp64": "f64", "fp32": "f32", "fp32x2": "f32x2"}[prec], "data": "synthetic",
         "config": cfg, "gpu_launches": launches,
         "roofline": dominant_roofline(prof, prec, peaks, hbm, hbm_src, jgroups or 1),
-        "kernel_rooflines": kernel_rooflines(prof, N_GRID, BATCH, peak, hbm, real_bytes, jgroups or 1),
+        "kernel_rooflines": kernel_rooflines(prof, N_GRID, BATCH, peak, hbm, real_bytes, jgroups or 1,
+                                             fx_peak_tflops(peaks)),
         "measured_peaks": dict(peaks, hbm_gbs=hbm, hbm_source=hbm_src),
         "e2e": {"value": world * BATCH / e2e_s, "unit": UNIT,
                 "h2d_bytes_per_step": int(params.nbytes + g.nbytes), "d2h_bytes_per_step": int(g.nbytes)},
@@ -1170,8 +1224,14 @@ def run_ours(args, world, rank, local):
             rec["speedup_vs_value"] = rec["value"] / value
             line["variants"][vp] = rec
         if prec == "fp64":
-            # the same FP64 path with the two-stage shared-memory transforms
-            # (LBO_OPT_KERNEL = 2) in place of the register kernels
+            # FP64 with FP64 transforms throughout: in registers
+            # (LBO_OPT_KERNEL = 1), and the two-stage shared-memory ones (2);
+            # the pairs of FP32 (1)
+            for vp, key in (("fp64", "fp64_register_transforms"), ("fp32x2", "fp32x2_pairs")):
+                rec = variant_leg(vp, tp, tg, tpc, tgc, stream, args.steps, peaks, hbm, ref, ref_c, rms, rms_c,
+                                  k_clean, kernel=1)
+                rec["speedup_vs_value"] = rec["value"] / value
+                line["variants"][key] = rec
             rec = variant_leg("fp64", tp, tg, tpc, tgc, stream, args.steps, peaks, hbm, ref, ref_c, rms, rms_c,
                               k_clean, kernel=2)
             rec["speedup_vs_value"] = rec["value"] / value
