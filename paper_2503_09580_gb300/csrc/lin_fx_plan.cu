@@ -76,9 +76,12 @@ lbo_status precompute_part(lbo_plan* p, const Tables& tb, const double* params, 
 // more than keeping a group in the L2 cache (N = 32, batch 256: 7.30 ms per
 // application at 64 MB, 6.40 at 143 MB, 5.74 at 572 MB, 5.58 at 1.1 GB, 5.54 at
 // 2.3 GB; N = 64, batch 64: 39.9, 39.8, 35.2, 32.9, 32.3).
-int group_size(const lbo_plan* p, int n) {
+int largest_group(const lbo_plan* p) {
   const size_t unit = (size_t)p->N * p->N * (p->N / 2 + 1) * sizeof(ci64) * p->J;
-  const int most = (int)std::max<size_t>(1, ((size_t)1 << 30) / unit);
+  return (int)std::max<size_t>(1, ((size_t)1 << 30) / unit);
+}
+int group_size(const lbo_plan* p, int n) {
+  const int most = largest_group(p);
   const int groups = (n + most - 1) / most;
   return (n + groups - 1) / groups;
 }
@@ -210,7 +213,10 @@ lbo_status run_linearized_fx(lbo_plan* p, const double* params, const double* g,
   fx::Tables tb;
   lbo_status st = fx::tables(p, &tb);
   const int part = fx::part_size(p, B), G = fx::group_size(p, part);
-  if (st == LBO_OK) st = fx::ensure(&p->ws, &p->ws_bytes, fx::workspace_bytes(p->N, part, G, p->J, !cached));
+  // the same buffer for cached and uncached calls and never more for a smaller
+  // batch: graphs captured with a plan keep its address
+  const size_t bytes = fx::workspace_bytes(p->N, part, std::min(part, fx::largest_group(p)), p->J, true);
+  if (st == LBO_OK) st = fx::ensure(&p->ws, &p->ws_bytes, bytes);
   const size_t n3 = (size_t)p->N * p->N * p->N;
   p->last_launches = 0;
   for (int b0 = 0; b0 < B && st == LBO_OK; b0 += part) {

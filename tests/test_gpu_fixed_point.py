@@ -134,3 +134,31 @@ def test_cut_off_changed_after_the_maxwellian_cache(n, precision):
         plain.apply_linearized(tp, tg, b)
         plan.sync(), plain.sync()
         assert torch.equal(a, b)
+
+
+def test_captured_graph_outlives_other_batches():
+    """A smaller batch, and an uncached call after a cached one, need no more
+    workspace than the larger, cached one: a graph captured with the plan still
+    replays.  1821 instances take two groups of 911, 1820 one group of 1820."""
+    n, L = 16, 8.0
+    params, g = workloads.batched_instances(n, L, batch=4, seed=130, noise=1e-3)
+    tp, tg = (torch.from_numpy(np.resize(x, (1821,) + x.shape[1:])).to(DEV) for x in (params, g))
+    plan = lbo.Plan(n, L, 0.5, n)
+    plan.cache_maxwellians(tp)
+    group = lbo.Group([plan], graph=True)
+    out, other = torch.empty_like(tg), torch.empty_like(tg[:1820])
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        for _ in range(2):  # eager, capture
+            group.apply_linearized([tp], [tg], [out])
+    torch.cuda.synchronize()
+    ref = out.clone()
+    plan.apply_linearized(tp[:1820].clone(), tg[:1820], other)
+    plan.sync()
+    out.zero_()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        group.apply_linearized([tp], [tg], [out])
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref) and torch.equal(other, ref[:1820])
+    group.close()
