@@ -18,9 +18,14 @@
 //   k_axis1_acc      InvFFT_1(sum_j phi_j FFT_1(psi^_j))
 //   k_combine_planes inverse axes 2 and 3 of L+, u and w, and L+ - u M - w g
 //
+// N = 32, 256 instances, J = 32: 5.7 ms (30.4 ms in FP64 registers, where the
+// FP64 pipe was the bound).  Arithmetic alone would take 2.3 to 2.8 ms at the
+// rate of register transforms, HBM 0.02 ms for inputs and outputs and about 1.5
+// for the spectra that pass between the kernels.
+//
 // Layout: half spectra [u][i1 or k1][k2][k3], all indices natural, k3 =
 // 0..N/2, ci64.  One thread transforms one pencil in registers (two threads,
-// joined by shuffles, for N = 48 and 64).
+// joined by shuffles, for N = 32, 48 and 64).
 #pragma once
 #include "fx64.cuh"
 #include "lin_kernels.cuh"
@@ -336,6 +341,10 @@ __global__ void __launch_bounds__(256) k_mh(const double* __restrict__ inst, con
 // sum.  One thread per pencil, the octant in shared memory; at N = 64, where
 // that takes 287 KB, a cluster of two blocks holds half of the planes d1 each
 // and reads the other's for axis 1.
+// Bound by latencies between its three passes (one block of (N/2+1)^2 pencils
+// holds the whole octant); N = 32, 256 instances: 0.60 ms, 3.0 in FP64.  At N =
+// 64 the pencils of 33 values spill 1 to 2 KB; a cluster of four instead of two
+// took 127 us where two take 98.
 // grid = (CL J, B), cluster CL, block = BLOCK, shared memory SMEM.
 template <int N>
 struct Octant {
@@ -485,6 +494,9 @@ __global__ void __launch_bounds__(Octant<N>::BLOCK) k_uhat(const double* __restr
 // EA[u]: the exponent of the products u^_j r^ of unit u, such that
 // sum(|re| + |im|) over every axis-1 pencil is at most 2^60; from the largest
 // sum over the bands of ub (k_uhat) times rm (k_axis1_head) over the columns.
+// Bands, not one bound per column: u^_j falls steeply, and the bits that one
+// bound of |u^_j| |r^| gives away are error.  Latency: 17 us at N = 32 for 86
+// instances, 9 us for 8.
 // grid = (J, B), block = 256.
 template <int N>
 __global__ void __launch_bounds__(256) k_unit_scale(const float* __restrict__ ub, const int* __restrict__ eU,
@@ -529,6 +541,9 @@ __global__ void __launch_bounds__(256) k_unit_scale(const float* __restrict__ ub
 // ------------------------------------------------------------ axis 1, inverse
 // W[u][i1][col] 2^EA[u] = InvFFT_1(u^_j r^).  The octant's entries carry the
 // shift from the column's exponent to EA, the data are not shifted.
+// Bound by load latency and issue: two threads per pencil and blocks of 64 put
+// 12 warps on an SM at N = 32.  256 instances: 0.92 ms, 4.3 in FP64; r^ kept in
+// registers over four nodes took as long (32.4 against 32.2 us per 7 instances).
 // grid = (ceil(NC T / 64), J, B), block = 64.
 template <int N>
 __global__ void __launch_bounds__(64) k_axis1_inv(const ci64* __restrict__ R, const int* __restrict__ eR,
@@ -760,6 +775,14 @@ __device__ __forceinline__ double plane_bound(float top, int E, int s) { return 
 // In place on W[u][i1]: psi <- M^h psi between the inverse and the forward
 // transforms of axes 2 and 3.  EP, BP [u][i1]: the plane's exponent and a bound
 // of its entries' values.
+// Bound by instruction issue (56 % of the slots at N = 32, integer pipe 55 %, 12
+// warps per SM) and instruction fetch.  The four passes are one loop around one
+// transform body: written out, 158 KB of code waited for instructions 46 % of
+// the time.  Two threads per pencil from N = 32 on, so that 168 registers and 12
+// warps per SM are enough: one thread per pencil took 105 us where this takes
+// 75.8 (7 instances), 16 warps of 128 registers 79.7.  A plane of 8, 16 or 32
+// threads stays within a warp and needs no block barrier.  256 instances: 2.54
+// ms, 15.2 in FP64; 5.5 TFLOP/s, 0.48 of the rate of register transforms.
 // grid = (N / PPC, J, B), block = Planes<N, PPC>::THREADS.
 template <int N, int PPC>
 __global__ void __launch_bounds__(Planes<N, PPC>::THREADS, Planes<N, PPC>::BLOCKS) k_plane(ci64* __restrict__ W, const int* __restrict__ EA,
@@ -858,7 +881,8 @@ __device__ __forceinline__ unsigned plane_umax(unsigned v, unsigned* slot) {
 // Axes 3 and 2 of FFT(r) (blockIdx.z = 0 with with_ratio; r = g/M with the
 // cut-off) or of FFT(g): F[z][b][i1][k2][k3], EP and BP [z][b][i1].  The field's plane is
 // read coalesced into shared memory as FP64, converted at the plane's own
-// exponent by the row threads.
+// exponent by the row threads.  Latency-bound: 0.19 ms for 256 instances at N =
+// 32 (1.4 in FP64).
 // grid = (N / PPC, B, 2 or 1), block = Planes<N, PPC>::THREADS.
 template <int N, int PPC>
 __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const double* __restrict__ field,
@@ -1083,6 +1107,9 @@ __device__ __forceinline__ int log2_above(double x) { return x > 0.0 ? ilogb(x) 
 // warp's shared memory, and the warps' sums at the end (integer sums: any
 // order gives the same result).  Then warp 0 transforms each column back, at
 // its own exponent EC[b][col].
+// Bound by issue and load latency; the sum over j stays on chip, where a launch
+// per node read and wrote it 32 times: 0.92 ms for 256 instances at N = 32, 4.5
+// in FP64.
 // grid = (ceil(NC T / 32), B), block = 32 WARPS, shared memory acc_smem(J).
 template <int N, int WARPS>
 constexpr size_t acc_smem(int J) {
@@ -1189,6 +1216,8 @@ __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict
 // A group of threads for each field transforms the block's planes of it, then
 // all threads combine.  Columns of F carry their own exponents EC[f][b][col];
 // they meet at the plane's largest.  NaN for a marked instance (bad).
+// The results become FP64 on the integer pipe (to_double).  Latency-bound: 0.33
+// ms for 256 instances at N = 32, 15 % of HBM; 1.0 in FP64.
 // grid = (N / PPC, B), block = FIELDS Planes<N, PPC>::THREADS.
 enum CombineMode { COMBINE, CACHED, FACTOR, QUAD };
 template <int N, int PPC, int MODE>
