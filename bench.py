@@ -66,6 +66,8 @@ KERNEL_SOURCES = {
     "f32_gain": ("lin_fused32.cu", "fused32.cuh", "tmem.cuh"),
 }
 NCU_TRAFFIC = {
+    # one capture of k_plane<32, 4> on 86 instances (a group of the benchmark workload): 789.2 MB read + 711.2 MB written
+    ("fx_plane_inv_mh_fwd", 32, "fp64"): (1500351232, "d0eb7cc965730afb"),
 }
 
 
