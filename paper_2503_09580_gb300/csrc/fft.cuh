@@ -102,6 +102,8 @@ static cudaError_t upload_twiddles_now() {
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_tw48_f, f48, sizeof(f48));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_tw48_ff, ff48, sizeof(ff48));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_tw48_dd, dd48, sizeof(dd48));
+  // in place before a kernel on a non-blocking stream reads them
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   return e;
 }
 

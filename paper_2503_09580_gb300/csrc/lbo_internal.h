@@ -102,6 +102,14 @@ struct lbo_solver {
 
 namespace lbo {
 lbo_status cuda_fail(cudaError_t e, const char* where);
+// A table from host memory, in place when this returns.  cudaMemcpy from pageable
+// memory may return while its last part is still on the way, and a kernel on a
+// non-blocking stream (a group's, a torch stream) is not ordered behind the
+// legacy stream that carries it.
+inline cudaError_t upload_table(void* dst, const void* src, size_t bytes) {
+  const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
 // learned preconditioner (network.cu)
 lbo_status network_correction(lbo_solver* S, const double* v, double* z);
 lbo_status network_record(lbo_solver* S, const double* w, const double* zk, double* s_scratch,

@@ -191,7 +191,7 @@ static lbo_status w_images(lbo_plan* p, const uint16_t** wf, const uint16_t** wi
       std::vector<uint16_t> img = w_image(p->N, d == 1, bf);
       cudaError_t e = cudaMalloc(&slot[d], img.size() * sizeof(uint16_t));
       if (e == cudaSuccess)
-        e = cudaMemcpy(slot[d], img.data(), img.size() * sizeof(uint16_t), cudaMemcpyHostToDevice);
+        e = upload_table(slot[d], img.data(), img.size() * sizeof(uint16_t));
       if (e != cudaSuccess) {
         for (int i = 0; i < 2; ++i)
           if (slot[i]) cudaFree(slot[i]), slot[i] = nullptr;
@@ -228,6 +228,7 @@ lbo_status run_linearized_dftmm(lbo_plan* p, const double* params, const double*
   if (!p->d_tc_err) {
     cudaError_t e = cudaMalloc(&p->d_tc_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(p->d_tc_err, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);  // as upload_table
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core error flag");
   }
   int* err = (int*)p->d_tc_err;
@@ -291,7 +292,7 @@ extern "C" lbo_status lbo_dft_axis_tensor(int N, int precision, int inverse, int
   lbo_status st = w_images(&tmp, &wf, &wi);
   int* err = nullptr;
   if (st == LBO_OK && cudaMalloc(&err, sizeof(int)) != cudaSuccess) st = LBO_ENOMEM;
-  if (st == LBO_OK) cudaMemset(err, 0, sizeof(int));
+  if (st == LBO_OK) cudaMemsetAsync(err, 0, sizeof(int), tmp.stream);
   int sms = 152, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

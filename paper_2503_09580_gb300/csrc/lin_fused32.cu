@@ -71,6 +71,8 @@ static cudaError_t upload_dct() {
     for (int d = 0; d < 8; ++d)
       t[k * 8 + d] = (float)((d == 0 ? 1.0 : 2.0) * std::cos(3.14159265358979323846 * k * d / 16.0));
   e = cudaMemcpyToSymbol(c_dct17, t, sizeof(t));
+  // in place before a kernel on a non-blocking stream reads it
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
   return e;
 }
@@ -551,6 +553,7 @@ lbo_status run_linearized_fused32(lbo_plan* p, const double* params, const doubl
   if (!p->d_tc_err) {
     e = cudaMalloc(&p->d_tc_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(p->d_tc_err, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);  // as upload_table
     if (e != cudaSuccess) return cuda_fail(e, "bounded-wait error flag");
   }
   FusedArgs a{};

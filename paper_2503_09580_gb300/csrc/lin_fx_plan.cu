@@ -148,7 +148,7 @@ lbo_status tables(lbo_plan* p, Tables* tb) {
       qe[j] = to_multipliers(x.data() + (size_t)j * Q, Q, inv_n3, buf.data() + (size_t)j * Q, pm + j);
     p->fx_omega_exp = to_multipliers(x.data() + words, Q, 1.0, buf.data() + words, nullptr);
     e = cudaMalloc(&p->d_fx, sizeof(long long) * buf.size());
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_fx, buf.data(), sizeof(long long) * buf.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload_table(p->d_fx, buf.data(), sizeof(long long) * buf.size());
     if (e != cudaSuccess) {
       free_fx_tables(p);
       return cuda_fail(e, "fixed-point tables");

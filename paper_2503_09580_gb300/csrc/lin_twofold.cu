@@ -69,7 +69,7 @@ void cos_pair(int N, long t, double* hi, double* lo) {
 template <typename T>
 lbo_status upload(const std::vector<T>& h, void** d) {
   cudaError_t e = cudaMalloc(d, sizeof(T) * h.size());
-  if (e == cudaSuccess) e = cudaMemcpy(*d, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload_table(*d, h.data(), sizeof(T) * h.size());
   if (e != cudaSuccess) {
     if (*d) cudaFree(*d);
     *d = nullptr;

@@ -267,7 +267,7 @@ std::vector<double> resample_matrix(int na, int nb, double L) {
 lbo_status upload_jobs(JobList& jl) {
   if (jl.host.empty()) return LBO_OK;
   cudaError_t e = cudaMalloc(&jl.dev, sizeof(RJob) * jl.host.size());
-  if (e == cudaSuccess) e = cudaMemcpy(jl.dev, jl.host.data(), sizeof(RJob) * jl.host.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload_table(jl.dev, jl.host.data(), sizeof(RJob) * jl.host.size());
   return e == cudaSuccess ? LBO_OK : cuda_fail(e, "mixed job list");
 }
 
@@ -447,8 +447,8 @@ lbo_status mixed_setup(lbo_solver* S, lbo_plan* const* plans, int nplans, const 
   };
   dalloc((void**)&M->d_N, sizeof(int) * M->nx);
   dalloc((void**)&M->d_off, sizeof(size_t) * M->nx);
-  if (e == cudaSuccess) e = cudaMemcpy(M->d_N, M->Nc.data(), sizeof(int) * M->nx, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(M->d_off, M->off.data(), sizeof(size_t) * M->nx, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload_table(M->d_N, M->Nc.data(), sizeof(int) * M->nx);
+  if (e == cudaSuccess) e = upload_table(M->d_off, M->off.data(), sizeof(size_t) * M->nx);
   // groups
   for (int p = 0; p < nplans; ++p) {
     Group G;
@@ -462,7 +462,7 @@ lbo_status mixed_setup(lbo_solver* S, lbo_plan* const* plans, int nplans, const 
     dalloc((void**)&G.in, sizeof(double) * cnt * n3);
     dalloc((void**)&G.out, sizeof(double) * cnt * n3);
     dalloc((void**)&G.params, sizeof(double) * cnt * 5);
-    if (e == cudaSuccess) e = cudaMemcpy(G.d_cells, G.cells.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload_table(G.d_cells, G.cells.data(), sizeof(int) * cnt);
     M->groups.push_back(G);
   }
   // resampling matrices for every ordered pair in use (the finest grid included)
@@ -499,9 +499,9 @@ lbo_status mixed_setup(lbo_solver* S, lbo_plan* const* plans, int nplans, const 
   }
   dalloc((void**)&M->mats64, sizeof(double) * mats.size());
   dalloc((void**)&M->mats32, sizeof(float) * mats32.size());
-  if (e == cudaSuccess) e = cudaMemcpy(M->mats64, mats.data(), sizeof(double) * mats.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload_table(M->mats64, mats.data(), sizeof(double) * mats.size());
   if (e == cudaSuccess)
-    e = cudaMemcpy(M->mats32, mats32.data(), sizeof(float) * mats32.size(), cudaMemcpyHostToDevice);
+    e = upload_table(M->mats32, mats32.data(), sizeof(float) * mats32.size());
   dalloc((void**)&M->tmp, sizeof(double) * 2 * cube * std::max<size_t>(njobs, 1));
   dalloc((void**)&M->nb2, sizeof(double) * 2 * M->len);
   dalloc((void**)&M->sweep_in, sizeof(double) * M->nx * nm3);
@@ -520,7 +520,7 @@ lbo_status mixed_setup(lbo_solver* S, lbo_plan* const* plans, int nplans, const 
     }
     double** dst = side == 0 ? &M->gL : &M->gR;
     dalloc((void**)dst, sizeof(double) * gh.size());
-    if (e == cudaSuccess) e = cudaMemcpy(*dst, gh.data(), sizeof(double) * gh.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload_table(*dst, gh.data(), sizeof(double) * gh.size());
   }
   if (e != cudaSuccess) return cuda_fail(e, "mixed set-up");
   lbo_status st = upload_jobs(M->transport);

@@ -450,7 +450,7 @@ static lbo_status upload_scales(NetState* ns) {
       return LBO_ENOMEM;
     }
   }
-  cudaError_t e = cudaMemcpy(ns->dev_sc, ns->scales, sizeof(float) * (CIN + COUT), cudaMemcpyHostToDevice);
+  cudaError_t e = upload_table(ns->dev_sc, ns->scales, sizeof(float) * (CIN + COUT));
   return e == cudaSuccess ? LBO_OK : cuda_fail(e, "network scales");
 }
 
@@ -660,11 +660,11 @@ lbo_status lbo_solver_train_network(lbo_solver* S, int hidden, int epochs, doubl
     set_error_text("network training allocation");
     result = LBO_ENOMEM;
   } else {
-    cudaMemcpy(d_sig, sig.data(), sizeof(float) * P, cudaMemcpyHostToDevice);
-    cudaMemcpy(d_sc, ns->scales, sizeof(float) * (CIN + COUT), cudaMemcpyHostToDevice);
-    cudaMemcpy(ns->theta, th0.data(), sizeof(float) * np, cudaMemcpyHostToDevice);
-    cudaMemset(m, 0, sizeof(float) * np);
-    cudaMemset(v, 0, sizeof(float) * np);
+    cudaMemsetAsync(m, 0, sizeof(float) * np, s);
+    cudaMemsetAsync(v, 0, sizeof(float) * np, s);
+    upload_table(d_sig, sig.data(), sizeof(float) * P);
+    upload_table(d_sc, ns->scales, sizeof(float) * (CIN + COUT));
+    upload_table(ns->theta, th0.data(), sizeof(float) * np);
     k_normalise<<<blocks_for(a), 256, 0, s>>>(ns->store_x, ns->store_t, P, nx, d_sig, d_sc, xn, tn);
     const float b1 = 0.9f, b2 = 0.999f;
     float c1 = 1.f, c2 = 1.f;
@@ -717,7 +717,7 @@ lbo_status lbo_solver_set_network(lbo_solver* S, int hidden, const float* params
   if (e == cudaSuccess && !ns->corr)
     e = cudaMalloc(&ns->corr, sizeof(float) * (size_t)S->nx * (COUT + (hidden > 0 ? hidden : 1)));
   if (e == cudaSuccess && !ns->feat) e = cudaMalloc(&ns->feat, sizeof(float) * (size_t)S->nx * CIN);
-  if (e == cudaSuccess) e = cudaMemcpy(ns->theta, params, sizeof(float) * np, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload_table(ns->theta, params, sizeof(float) * np);
   if (e != cudaSuccess) return cuda_fail(e, "set network");
   std::memcpy(ns->scales, scales, sizeof(ns->scales));
   lbo_status st = upload_scales(ns);

@@ -129,8 +129,8 @@ lbo_status ensure_omega_quadrature(lbo_plan* p, QuadState* qs) {
   if (e == cudaSuccess) e = cudaMalloc(&d_w, sizeof(double) * wjm.size());
   if (e == cudaSuccess) e = cudaMalloc(&d_out, sizeof(double) * H);
   if (e == cudaSuccess) e = cudaMalloc(&qs->d_omq, rb * H);
-  if (e == cudaSuccess) e = cudaMemcpy(d_fac, fac.data(), sizeof(double2) * fac.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_w, wjm.data(), sizeof(double) * wjm.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload_table(d_fac, fac.data(), sizeof(double2) * fac.size());
+  if (e == cudaSuccess) e = upload_table(d_w, wjm.data(), sizeof(double) * wjm.size());
   if (e == cudaSuccess) {
     const double scale = 16.0 * pi * pi / ((double)N * N * N);
     const int grid = (int)std::min<size_t>((H + 255) / 256, 152 * 8);
@@ -240,7 +240,7 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
         h.insert(h.end(), w, w + 2);
       }
       e = cudaMalloc(&qs->d_gsw, sizeof(double) * h.size());
-      if (e == cudaSuccess) e = cudaMemcpy(qs->d_gsw, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = upload_table(qs->d_gsw, h.data(), sizeof(double) * h.size());
       if (e != cudaSuccess) return cuda_fail(e, "quadrature nodes upload");
       qs->gsw_p = qs->p;
       qs->gsw_plan_tables = p->d_phi32;

@@ -1085,8 +1085,8 @@ lbo_status lbo_solver_create(const lbo_problem* pb, lbo_plan* plan, lbo_solver**
       S->kL = pb->bc_left == LBO_BC_WALL ? std::sqrt(2.0 * 3.141592653589793 / pb->wall_left[0]) : 0.0;
       S->kR = pb->bc_right == LBO_BC_WALL ? std::sqrt(2.0 * 3.141592653589793 / pb->wall_right[0]) : 0.0;
     }
-    cudaError_t e = cudaMemcpy(S->WL, wl.data(), sizeof(double) * S->n3, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(S->WR, wr.data(), sizeof(double) * S->n3, cudaMemcpyHostToDevice);
+    cudaError_t e = upload_table(S->WL, wl.data(), sizeof(double) * S->n3);
+    if (e == cudaSuccess) e = upload_table(S->WR, wr.data(), sizeof(double) * S->n3);
     if (e != cudaSuccess) {
       lbo_solver_destroy(S);
       return cuda_fail(e, "solver tables");

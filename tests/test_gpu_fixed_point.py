@@ -162,3 +162,23 @@ def test_captured_graph_outlives_other_batches():
     torch.cuda.synchronize()
     assert torch.equal(out, ref) and torch.equal(other, ref[:1820])
     group.close()
+
+
+@pytest.mark.parametrize("n,precision,kernel", [(16, "fp64", 0), (64, "fp64", 0), (32, "fp64", 1), (32, "fp32", 0),
+                                                (16, "fp64x2", 0)])
+def test_first_application_on_a_non_blocking_stream(n, precision, kernel):
+    """The tables a plan makes at its first application are in place before
+    the kernels of a stream that is not ordered behind the legacy one."""
+    L = 8.0
+    params, g = workloads.batched_instances(n, L, batch=2, seed=140, noise=0.0)
+    tp, tg = torch.from_numpy(params).to(DEV), torch.from_numpy(g).to(DEV)
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(4):
+        plan = lbo.Plan(n, L, 0.5, n, hemisphere_p=2, precision=precision, kernel=kernel, q_sinc_quadrature=1)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            outs.append([plan.apply_linearized(tp, tg, torch.empty_like(tg)),
+                         plan.apply_quadratic(tg, torch.empty_like(tg))])
+            plan.sync()
+    for lin, quad in outs[1:]:
+        assert torch.equal(lin, outs[0][0]) and torch.equal(quad, outs[0][1])

@@ -5,6 +5,7 @@ the mixed-N solver against the oracle's FFT-based resampling, and the
 register-resident 32-point transform of the FP64 kernels against a direct
 DFT."""
 import os
+import re
 import shutil
 import subprocess
 
@@ -89,3 +90,25 @@ def test_fixed_point_arithmetic_against_long_double(tmp_path):
             assert err < 1.5 * 20 ** 0.5 and abs(bias) < (0.25 if n == 24 else 0.02), (n, d, err, bias)
     for h in (8, 12, 16, 24, 32):
         assert res["dct%d" % h][0] < 2 * 1.5 * h / 2, h
+
+
+def test_tables_are_uploaded_in_order_with_every_stream():
+    """Outside the plan's build_tables, which ends with a device
+    synchronisation, no source copies or clears a table on the legacy stream
+    without waiting for it: kernels of a non-blocking stream would not be
+    ordered behind it."""
+    csrc = os.path.join(ROOT, "paper_2503_09580_gb300", "csrc")
+    found = []
+    for name in sorted(os.listdir(csrc)):
+        if not name.endswith((".cu", ".cuh", ".h")) or name == "lbo.cu":
+            continue
+        with open(os.path.join(csrc, name)) as fh:
+            text = fh.read()
+        for call in re.finditer(r"cudaMemcpy\([^;]*cudaMemcpyHostToDevice\)|cudaMemcpyToSymbol\(|cudaMemset\(", text):
+            if "cudaStreamSynchronize(cudaStreamLegacy)" not in text[call.start():call.start() + 1200]:
+                found.append((name, call.group(0)))
+    assert not found
+    with open(os.path.join(csrc, "lbo.cu")) as fh:
+        text = fh.read()
+    assert not re.search(r"HostToDevice", text[text.index("build_phit(lbo_plan* p, const double* d_stab, T* d_phit) {"):])
+    assert "cudaDeviceSynchronize()" in text[text.index("static lbo_status build_phit(lbo_plan* p, const double* d_stab, T* d_phit) {"):]
