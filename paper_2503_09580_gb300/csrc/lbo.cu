@@ -192,6 +192,7 @@ static lbo_status build_tables(lbo_plan* p) {
     return s2;
   }
   p->tables_dirty = false;
+  p->tables_made += 1;
   p->mc_valid = false;
   return LBO_OK;
 }

@@ -16,6 +16,7 @@ struct lbo_plan {
   int q_sinc_quad = 0;  // Q's loss multiplier: 1 = the hemisphere quadrature of Eq. (2.16)
   cudaStream_t stream = nullptr;
   bool tables_dirty = false;
+  int tables_made = 0;  // how often the tables were built: what derives from the radial rule is keyed by it
   // radial rule (host copy)
   std::vector<double> gj, wj, Bj;
   // device tables of Algorithm 1

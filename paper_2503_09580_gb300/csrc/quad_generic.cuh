@@ -33,12 +33,12 @@ struct QuadState {
   // transform precision of omq_prec, for hemisphere order omq_p
   void* d_omq = nullptr;
   int omq_prec = -1, omq_p = -1;
-  const void* omq_tables = nullptr;
+  int omq_tables = 0;  // lbo_plan::tables_made
   void* ws = nullptr;
   size_t ws_bytes = 0;
   double* d_gsw = nullptr;      // device copy: radial nodes, sigma, w_m (fused path)
   int gsw_p = -1;
-  const void* gsw_plan_tables = nullptr;
+  int gsw_tables = 0;
 };
 
 template <int N>

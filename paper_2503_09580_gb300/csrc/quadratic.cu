@@ -99,7 +99,7 @@ __global__ void k_to_transform_type(const double* __restrict__ a, T* __restrict_
 // the precision, the hemisphere rule or the tables change.
 lbo_status ensure_omega_quadrature(lbo_plan* p, QuadState* qs) {
   const int prec = uses_fixed_point(p) ? (int)LBO_PREC_FP64 : p->precision;  // fixed point converts it from FP64
-  if (qs->d_omq && qs->omq_prec == prec && qs->omq_p == qs->p && qs->omq_tables == (const void*)p->d_phi64)
+  if (qs->d_omq && qs->omq_prec == prec && qs->omq_p == qs->p && qs->omq_tables == p->tables_made)
     return LBO_OK;
   if (qs->d_omq) cudaFree(qs->d_omq);
   qs->d_omq = nullptr;
@@ -162,7 +162,7 @@ lbo_status ensure_omega_quadrature(lbo_plan* p, QuadState* qs) {
   }
   qs->omq_prec = prec;
   qs->omq_p = qs->p;
-  qs->omq_tables = p->d_phi64;
+  qs->omq_tables = p->tables_made;
   return LBO_OK;
 }
 
@@ -224,7 +224,7 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
   }
   {
     // radial nodes, hemisphere nodes and weights on the device
-    if (qs->gsw_p != qs->p || qs->gsw_plan_tables != (const void*)p->d_phi32) {
+    if (!qs->d_gsw || qs->gsw_p != qs->p || qs->gsw_tables != p->tables_made) {
       if (qs->d_gsw) cudaFree(qs->d_gsw);
       qs->d_gsw = nullptr;
       std::vector<double> h(p->gj);
@@ -243,7 +243,7 @@ lbo_status apply_quadratic_device(lbo_plan* p, const double* f, double* out, int
       if (e == cudaSuccess) e = upload_table(qs->d_gsw, h.data(), sizeof(double) * h.size());
       if (e != cudaSuccess) return cuda_fail(e, "quadrature nodes upload");
       qs->gsw_p = qs->p;
-      qs->gsw_plan_tables = p->d_phi32;
+      qs->gsw_tables = p->tables_made;
     }
   }
   if (fused) {

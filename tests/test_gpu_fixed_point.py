@@ -182,3 +182,22 @@ def test_first_application_on_a_non_blocking_stream(n, precision, kernel):
             plan.sync()
     for lin, quad in outs[1:]:
         assert torch.equal(lin, outs[0][0]) and torch.equal(quad, outs[0][1])
+
+
+@pytest.mark.parametrize("opts", [{}, {"q_sinc_quadrature": 1}, {"precision": "fp32"}, {"kernel": 1}])
+def test_radial_cut_and_scale_changed_after_an_application(opts):
+    """R and C set after Q and L have run on a plan: everything derived from
+    the radial rule is made again, equal to a new plan's."""
+    n, L = 32, 8.0
+    params, g = workloads.batched_instances(n, L, batch=2, seed=153, noise=0.0)
+    opts = dict(opts, hemisphere_p=2)
+    plan = lbo.Plan(n, L, 0.5, n, **opts)
+    now = {"R": 4 * L / (3 + np.sqrt(2.0)), "C": 1 / (4 * np.pi)}
+    for key, factor in (("R", 1.0), ("R", 0.6), ("C", 1 / 64), ("C", 64.0), ("R", 1 / 0.6)):
+        now[key] *= factor
+        plan.set(key, now[key])
+        new = lbo.Plan(n, L, 0.5, n, **opts)
+        for k, v in now.items():
+            new.set(k, v)
+        for quad in (True, False):
+            assert np.array_equal(apply(plan, params, g, quad=quad), apply(new, params, g, quad=quad)), (key, factor)
