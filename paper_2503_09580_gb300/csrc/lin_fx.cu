@@ -29,13 +29,13 @@ struct Buffers {
   // of B instances
   ci64 *R, *F, *MH;  // r^; fields L+, u, w (first: FFT(r), FFT(g) of the planes); M's factors
   i64* mh;
-  double *inst, *BPh;
-  float *rm, *ub;
+  double* inst;
+  float *rm, *ub, *BPh;
   int *eR, *em, *eM, *EPh, *EC, *bad;
   // of G instances
   ci64* W;
   i64* U;
-  double* BP;
+  float* BP;
   int *eU, *EA, *EP;
   size_t bytes;
   Buffers(void* base, size_t B, size_t G, size_t J, bool own_u) {

@@ -768,13 +768,14 @@ __device__ __forceinline__ void store_spectrum(const ci64 (&x)[Geo<N>::V], const
   }
 }
 
-// a bound of a plane's entries' values: twice (the packed pair's sum) the
-// largest pencil sum `top` 2^32 at the exponent before the shift s
-__device__ __forceinline__ double plane_bound(float top, int E, int s) { return scalbn((double)top, 33 + E - s); }
+// a bound of a plane's entries in its own units: twice (the packed pair's sum)
+// the largest pencil sum `top` 2^32 at the exponent before the shift s; at least
+// 2^60 and below 2^61, whatever the exponent
+__device__ __forceinline__ float plane_bound(float top, int s) { return scalbnf(top, 33 - s); }
 
 // In place on W[u][i1]: psi <- M^h psi between the inverse and the forward
 // transforms of axes 2 and 3.  EP, BP [u][i1]: the plane's exponent and a bound
-// of its entries' values.
+// of its entries, |entry| <= BP 2^EP.
 // Bound by instruction issue (56 % of the slots at N = 32, integer pipe 55 %, 12
 // warps per SM) and instruction fetch.  The four passes are one loop around one
 // transform body: written out, 158 KB of code waited for instructions 46 % of
@@ -788,7 +789,7 @@ template <int N, int PPC>
 __global__ void __launch_bounds__(Planes<N, PPC>::THREADS, Planes<N, PPC>::BLOCKS) k_plane(ci64* __restrict__ W, const int* __restrict__ EA,
                                                                  const i64* __restrict__ mh,
                                                                  const int* __restrict__ em, int* __restrict__ EP,
-                                                                 double* __restrict__ BP) {
+                                                                 float* __restrict__ BP) {
   constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, V = Geo<N>::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned red[4 * PPC];
@@ -860,7 +861,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS, Planes<N, PPC>::BLOCK
   store_spectrum<N>(x, t, gw);
   if (t.tp == 0) {
     EP[u * N + i1] = E;
-    BP[u * N + i1] = plane_bound(top, E, s);
+    BP[u * N + i1] = plane_bound(top, s);
   }
 }
 
@@ -888,7 +889,7 @@ template <int N, int PPC>
 __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const double* __restrict__ field,
                                                                       const double* __restrict__ inst, int with_ratio, int cutoff,
                                                                       ci64* __restrict__ F, int* __restrict__ EP,
-                                                                      double* __restrict__ BP, int* __restrict__ bad) {
+                                                                      float* __restrict__ BP, int* __restrict__ bad) {
   constexpr int NC = Geo<N>::NC, V = Geo<N>::V, TPP = Geo<N>::TPP, RS = N + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned red[3 * PPC];
@@ -954,7 +955,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
   store_spectrum<N>(x, t, F + (u * N + i1) * NC);
   if (t.tp == 0) {
     EP[u * N + i1] = E;
-    BP[u * N + i1] = plane_bound(sum, E, s);
+    BP[u * N + i1] = plane_bound(sum, s);
   }
 }
 
@@ -1099,9 +1100,11 @@ __device__ __forceinline__ int log2_above(double x) { return x > 0.0 ? ilogb(x) 
 //
 // The exponent EL of L^+ and the right shift sp of every plane of every node
 // into units where phi_j x / 2^64 carries EL: with S_j the sum over planes of
-// the bounds BP (an axis-1 pencil of psi^_j at most), S_j <= 2^60 of those
+// the bounds BP 2^EP (an axis-1 pencil of psi^_j at most), S_j <= 2^60 of those
 // units and sum_j S_j max|phi_j| <= 2^61 of EL's.  q[j], pm[j]: the exponent and
-// the largest value of the multipliers phi_j.
+// the largest value of the multipliers phi_j.  S_j is kept as a value and the
+// largest exponent of its planes: as one FP64 number it overflowed, unlike the
+// result, for inputs 2^20 below FP64's own limit.
 //
 // Warp w takes the nodes j = w, w + WARPS, ...; their phi_j psi^_j add up in the
 // warp's shared memory, and the warps' sums at the end (integer sums: any
@@ -1113,17 +1116,18 @@ __device__ __forceinline__ int log2_above(double x) { return x > 0.0 ? ilogb(x) 
 // grid = (ceil(NC T / 32), B), block = 32 WARPS, shared memory acc_smem(J).
 template <int N, int WARPS>
 constexpr size_t acc_smem(int J) {
-  return sizeof(ci64) * WARPS * Geo<N>::V * 32 + (sizeof(double) + sizeof(int) * N) * (size_t)J;
+  return sizeof(ci64) * WARPS * Geo<N>::V * 32 + (sizeof(double) + sizeof(int) * (N + 1)) * (size_t)J;
 }
 template <int N, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict__ W, const int* __restrict__ EP,
-                                                        const double* __restrict__ BP, const i64* __restrict__ phi,
+                                                        const float* __restrict__ BP, const i64* __restrict__ phi,
                                                         const int* __restrict__ q, const double* __restrict__ pm,
                                                         ci64* __restrict__ F, int* __restrict__ EC, int J) {
   constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, T = Geo<N>::T, V = Geo<N>::V, Q = 3 * (N / 2) * (N / 2) + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* part = (double*)(smem_raw + sizeof(ci64) * WARPS * V * 32);  // [J] S_j max|phi_j|
-  int* sp = (int*)(part + J);                                         // [J][N]
+  int* pe = (int*)(part + J);                                         // [J] the exponents of part
+  int* sp = pe + J;                                                   // [J][N]
   __shared__ int el;
   const int b = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int id = blockIdx.x * 32 + lane, h = T == 2 ? id & 1 : 0;
@@ -1133,23 +1137,31 @@ __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict
   if (threadIdx.x == 0) el = kZeroExp;
   __syncthreads();
   for (int j = w; j < J; j += WARPS) {
+    const size_t u = ((size_t)b * J + j) * N;
+    int base = EP[u + lane % N];
+    for (int i = lane + 32; i < N; i += 32) base = max(base, EP[u + i]);
+    base = __reduce_max_sync(0xffffffffu, base);
     double s = 0.0;
-    for (int i = lane; i < N; i += 32) s += BP[((size_t)b * J + j) * N + i];
+    for (int i = lane; i < N; i += 32) s += BP[u + i] * exp2_neg(base - EP[u + i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
       part[j] = s * pm[j];
-      atomicMax(&el, log2_above(s) - kSumBits - q[j] + 64);
+      pe[j] = base;
+      atomicMax(&el, base + log2_above(s) - kSumBits - q[j] + 64);
     }
   }
   __syncthreads();
   if (w == 0) {
+    int base = pe[lane % J];
+    for (int j = lane + 32; j < J; j += 32) base = max(base, pe[j]);
+    base = __reduce_max_sync(0xffffffffu, base);
     double s = 0.0;
-    for (int j = lane; j < J; j += 32) s += part[j];
+    for (int j = lane; j < J; j += 32) s += scalbn(part[j], pe[j] - base);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
-      const int e = max(el, log2_above(s * 1.0001) - 61);
+      const int e = max(el, base + log2_above(s * 1.0001) - 61);
       el = e < kZeroExp / 2 ? 0 : e;
     }
   }

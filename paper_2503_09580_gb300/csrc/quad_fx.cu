@@ -45,8 +45,7 @@ struct Cut {
 struct Buffers {
   ci64 *R, *F, *PW, *Z, *tab1, *tab;
   i64 *accG, *om3;
-  double *BPh, *BP;
-  float* rm;
+  float *rm, *BPh, *BP;
   int *eR, *EF, *EPh, *EC, *bad, *EP, *accE;
   size_t bytes;
   Buffers(void* base, size_t B, size_t J, const QuadRule& r, const Cut& c) {

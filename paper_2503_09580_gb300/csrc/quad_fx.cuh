@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
                                                             int J, int mc, int bj0, int first, int last, int guard, int ke,
                                                             i64* __restrict__ accG, int* __restrict__ accE,
                                                             ci64* __restrict__ PW, int* __restrict__ EP,
-                                                            double* __restrict__ BP) {
+                                                            float* __restrict__ BP) {
   using G = GeoQ<N>;
   constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC, T = Geo<N>::T, V = Geo<N>::V, TPP = G::TPP, RS = G::RS, FT = Geo<N>::TPP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
   store_spectrum<N>(x, t, PW + ((size_t)bj * N + i1) * NC);
   if (tp == 0) {
     EP[(size_t)bj * N + i1] = E;
-    BP[(size_t)bj * N + i1] = plane_bound(top, E, s);
+    BP[(size_t)bj * N + i1] = plane_bound(top, s);
   }
 }
 

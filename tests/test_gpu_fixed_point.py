@@ -201,3 +201,29 @@ def test_radial_cut_and_scale_changed_after_an_application(opts):
             new.set(k, v)
         for quad in (True, False):
             assert np.array_equal(apply(plan, params, g, quad=quad), apply(new, params, g, quad=quad)), (key, factor)
+
+
+@pytest.mark.parametrize("n", [16, 32, 64])
+def test_up_to_the_limits_of_fp64(n):
+    """Powers of two on the input are exact up to FP64's own limits: as long
+    as r = g/M is finite for L[g], and the two terms of Q(f,f) for Q (the
+    result 2^8 below the largest number).  The bounds of intermediate fields,
+    which carry the N^3 of unnormalised transforms, reach beyond.  An r that
+    is not finite gives NaN in its own instance."""
+    L, theta = 8.0, 2.0
+    params = np.array([[1.0, 0.1, -0.2, 0.05, theta]] * 2)
+    d = [workloads.velocity_axis(n, L) - u for u in params[0, 1:4]]
+    d2 = d[0][:, None, None] ** 2 + d[1][None, :, None] ** 2 + d[2][None, None, :] ** 2
+    g = np.stack([(2 * np.pi * theta) ** -1.5 * np.exp(-d2 / (2 * theta)) * (1 + c * d[0][:, None, None])
+                  for c in (0.3, 0.2)])
+    plan = lbo.Plan(n, L, 0.5, n, hemisphere_p=2)
+    base = apply(plan, params, g)
+    for e in (960, 1013, 1020):
+        assert np.array_equal(apply(plan, params, np.ldexp(g, e)), np.ldexp(base, e)), e
+    out = apply(plan, params, np.stack([np.ldexp(g[0], 1000), np.ldexp(g[1], 1024)]))
+    assert np.array_equal(out[0], np.ldexp(base[0], 1000)) and np.all(np.isnan(out[1]))
+    base = apply(plan, params, g, quad=True)
+    top = int(np.log2(np.abs(base).max())) + 1
+    for margin in (60, 20, 12, 8):
+        e = (1023 - top - margin) // 2
+        assert np.array_equal(apply(plan, params, np.ldexp(g, e), quad=True), np.ldexp(base, 2 * e)), margin
