@@ -70,3 +70,25 @@ def test_every_linearized_launch_has_a_roofline_model():
             assert bench.kernel_bytes_per_instance(n, 32, 8) > 0, n
         else:
             assert bench.kernel_flops_per_instance(n, 32) > 0, n
+
+
+def test_the_printed_line_stays_short():
+    """stdout carries the headline alone, below 3 KB, however many kernels,
+    variants and workloads the record holds: the line was 37 KB once, and
+    whoever kept the last 3 KB of the output could not read it."""
+    bench = _bench_module()
+    cfg = bench.workload_config(0.5, "fp64")
+    cfg.update({k: "x" * n for k, n in (("eps", 8), ("jgroups", 5), ("transforms", 110), ("planes_per_cta", 5),
+                                        ("parallelism", 44), ("l2", 60))})
+    report = {"rel_err_vs_oracle": 1.2345678901234e-13, "bound": 1.2345678901234e-13, "text": "x" * 220}
+    line = dict({k: 1.2345678901234567 for k in bench.HEADLINE_KEYS}, metric=bench.METRIC, unit=bench.UNIT, config=cfg,
+                roofline={"kernel": "x" * 30, "text": "x" * 450}, measured_peaks={"text": "x" * 190},
+                e2e={"text": "x" * 110}, clocks={"text": "x" * 110}, accuracy_noisy=report, accuracy_noise_free=report,
+                variants={"a": "x" * 20000}, kernels={"b": "x" * 600})
+    short = bench.headline(line)
+    assert len(json.dumps(short)) < 3000
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "gpu_launches", "roofline", "e2e", "clocks"):
+        assert short[key] == line[key]
+    with open(os.path.join(ROOT, "bench.py")) as fh:
+        assert "print(json.dumps(line), flush=True)" not in fh.read().split("def run_ours")[1]
