@@ -26,9 +26,9 @@ constexpr int ACC_WARPS = 8, PPC = PlanesPPC<N>::v, CPPC = CombinePPC<N>::v;
 // How a call is cut: G instances at a time whose J plane spectra PW stay below
 // 512 MB; of a pair's hemisphere nodes as many classes per launch as keep their
 // Z and the table of e_2 e_3 below 1 GB each, and of the (instance, radial node)
-// pairs as many as 1 GB of Z holds.
+// pairs as many as 1 GB of Z holds, spread evenly over the launches.
 struct Cut {
-  int G, classes, nodes, pairs;  // nodes: the most of a launch
+  int G, classes, nodes, most, pairs;  // nodes, most: the most nodes and pairs of a launch
   Cut(int B, int J, const QuadRule& r) {
     const size_t z = 2 * sizeof(ci64) * H, gb = (size_t)1 << 30;
     G = (int)std::min<size_t>(B, std::max<size_t>(1, (gb / 2) / (sizeof(ci64) * H * J)));
@@ -36,12 +36,15 @@ struct Cut {
     for (int c = 0; c < r.classes; ++c) wide = std::max(wide, r.class_begin[c + 1] - r.class_begin[c]);
     classes = (int)std::min<size_t>(r.classes, std::max<size_t>(1, std::min(gb / z, gb / (sizeof(ci64) * NC * J * wide))));
     nodes = std::min(r.M, classes * wide);
-    const size_t all = (size_t)G * J, most = std::min<size_t>(all, std::max<size_t>(1, gb / (z * classes)));
+    const size_t all = (size_t)G * J;
+    most = (int)std::min<size_t>(all, std::max<size_t>(1, gb / (z * classes)));
     const size_t launches = (all + most - 1) / most;
     pairs = (int)((all + launches - 1) / launches);
   }
 };
 
+// Sized by the most pairs of a launch, not by the even share: a smaller batch
+// never needs more, so what was captured with a larger one keeps its buffer.
 struct Buffers {
   ci64 *R, *F, *PW, *Z, *tab1, *tab;
   i64 *accG, *om3;
@@ -58,10 +61,10 @@ struct Buffers {
     take(R, B * H);
     take(F, 2 * B * H);
     take(PW, c.G * J * H);
-    take(Z, (size_t)c.pairs * c.classes * 2 * H);
+    take(Z, (size_t)c.most * c.classes * 2 * H);
     take(tab1, J * c.classes * N);
     take(tab, J * c.nodes * NC);
-    take(accG, rest ? c.pairs * n3 : 0);
+    take(accG, rest ? c.most * n3 : 0);
     take(om3, r.omega3 ? H : 0);
     take(BPh, B * N);
     take(BP, c.G * J * N);
@@ -72,7 +75,7 @@ struct Buffers {
     take(EC, 2 * B * NC);
     take(bad, B);
     take(EP, c.G * J * N);
-    take(accE, rest ? (size_t)c.pairs * N * N : 0);
+    take(accE, rest ? (size_t)c.most * N * N : 0);
     bytes = (size_t)(p - (unsigned char*)base);
   }
 };

@@ -112,3 +112,17 @@ def test_tables_are_uploaded_in_order_with_every_stream():
         text = fh.read()
     assert not re.search(r"HostToDevice", text[text.index("build_phit(lbo_plan* p, const double* d_stab, T* d_phit) {"):])
     assert "cudaDeviceSynchronize()" in text[text.index("static lbo_status build_phit(lbo_plan* p, const double* d_stab, T* d_phit) {"):]
+
+
+def test_fixed_point_workspaces_do_not_shrink_with_the_batch(tmp_path):
+    """Q's fixed-point workspace, from the library itself: a smaller batch never
+    needs a larger buffer, so a graph captured with one batch keeps its buffer
+    when the plan is called with another."""
+    lib = os.path.join(ROOT, "paper_2503_09580_gb300", "_lib")
+    if not os.path.exists(os.path.join(lib, "liblbo.so")) or not os.path.exists(NVCC):
+        pytest.skip("library or nvcc not available")
+    exe = str(tmp_path / "fx_workspace")
+    subprocess.check_call([NVCC, "-std=c++17", "-O1", "-o", exe, os.path.join(HOST, "fx_workspace.cu"), "-L" + lib,
+                           "-llbo", "-Xlinker", "-rpath=" + lib])
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.startswith("ok"), r.stdout
