@@ -288,7 +288,9 @@ __global__ void __launch_bounds__(kInstanceThreads<N>) k_instance(const double* 
   __syncthreads();
   if (t >= TH && t < TH + N) {
     const double m = (e * __longlong_as_double((i64)top[1])) * __longlong_as_double((i64)top[2]);
-    em1[b * N + ti] = m > 0.0 && isfinite(m) ? ilogb(m) - 59 : 0;
+    // a plane where every entry underflows has no magnitude: its bound must not
+    // set the exponent of the sum over the planes
+    em1[b * N + ti] = !(m > 0.0) ? kZeroExp : (isfinite(m) ? ilogb(m) - 59 : 0);
   }
 }
 

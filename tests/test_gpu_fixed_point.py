@@ -227,3 +227,19 @@ def test_up_to_the_limits_of_fp64(n):
     for margin in (60, 20, 12, 8):
         e = (1023 - top - margin) // 2
         assert np.array_equal(apply(plan, params, np.ldexp(g, e), quad=True), np.ldexp(base, 2 * e)), margin
+
+
+@pytest.mark.parametrize("n,theta,rho", [(32, 0.05, 1.0), (32, 0.05, 1e-40), (16, 0.05, 1e-100), (32, 0.07, 1e-100)])
+def test_cold_thin_gases_whose_outer_planes_vanish(n, theta, rho):
+    """exp(-|v - u|^2 / theta) underflows on the outer planes of a cold gas;
+    they have no part in the exponents of the others, however small rho is."""
+    L = 8.0
+    params = np.array([[rho, 0.1, -0.2, 0.05, theta]])
+    d = [workloads.velocity_axis(n, L) - u for u in params[0, 1:4]]
+    assert (np.exp(-d[0] ** 2 / theta) == 0).any()
+    d2 = d[0][:, None, None] ** 2 + d[1][None, :, None] ** 2 + d[2][None, None, :] ** 2
+    g = (rho * (2 * np.pi * theta) ** -1.5 * np.exp(-d2 / (2 * theta)) * (1 + 0.3 * d[0][:, None, None] + d2))[None]
+    a = apply(lbo.Plan(n, L, 0.5, n), params, g)
+    b = apply(lbo.Plan(n, L, 0.5, n, kernel=1), params, g)
+    tol = 2 * 4 * U64 * max(ratio_rms(params, g, n, L)[0], 64.0)
+    assert np.abs(a - b).max() <= tol * np.abs(b).max()
