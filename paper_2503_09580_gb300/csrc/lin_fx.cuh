@@ -1140,11 +1140,20 @@ __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict
   __syncthreads();
   for (int j = w; j < J; j += WARPS) {
     const size_t u = ((size_t)b * J + j) * N;
-    int base = EP[u + lane % N];
-    for (int i = lane + 32; i < N; i += 32) base = max(base, EP[u + i]);
+    constexpr int R = (N + 31) / 32;  // planes per lane
+    int e[R], base = kZeroExp;
+    float f[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = lane + 32 * r;
+      e[r] = i < N ? EP[u + i] : 2 * kZeroExp;
+      f[r] = i < N ? BP[u + i] : 0.f;
+      base = max(base, e[r]);
+    }
     base = __reduce_max_sync(0xffffffffu, base);
     double s = 0.0;
-    for (int i = lane; i < N; i += 32) s += BP[u + i] * exp2_neg(base - EP[u + i]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) s += f[r] * exp2_neg(base - e[r]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
