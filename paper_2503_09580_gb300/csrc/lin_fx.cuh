@@ -770,10 +770,12 @@ __device__ __forceinline__ void store_spectrum(const ci64 (&x)[Geo<N>::V], const
   }
 }
 
-// a bound of a plane's entries in its own units: twice (the packed pair's sum)
-// the largest pencil sum `top` 2^32 at the exponent before the shift s; at least
-// 2^60 and below 2^61, whatever the exponent
-__device__ __forceinline__ float plane_bound(float top, int s) { return scalbnf(top, 33 - s); }
+// a bound of a plane's entries in its own units: twice (the packed pair's sum) the
+// largest pencil sum `top` 2^32, after the shift that brings it to [2^59, 2^60) and
+// the halving of the plane's unit: the bits of `top` at the exponent 60
+__device__ __forceinline__ float plane_bound(float top) {
+  return __uint_as_float((__float_as_uint(top) & 0x7fffffu) | (127u + 60u) << 23);
+}
 
 // In place on W[u][i1]: psi <- M^h psi between the inverse and the forward
 // transforms of axes 2 and 3.  EP, BP [u][i1]: the plane's exponent and a bound
@@ -863,7 +865,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS, Planes<N, PPC>::BLOCK
   store_spectrum<N>(x, t, gw);
   if (t.tp == 0) {
     EP[u * N + i1] = E;
-    BP[u * N + i1] = plane_bound(top, s);
+    BP[u * N + i1] = plane_bound(top);
   }
 }
 
@@ -957,7 +959,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
   store_spectrum<N>(x, t, F + (u * N + i1) * NC);
   if (t.tp == 0) {
     EP[u * N + i1] = E;
-    BP[u * N + i1] = plane_bound(sum, s);
+    BP[u * N + i1] = plane_bound(sum);
   }
 }
 
@@ -1097,6 +1099,8 @@ __global__ void __launch_bounds__(64) k_axis1_head(ci64* __restrict__ F, const i
 
 // ------------------------------------------------------------ accumulation
 __device__ __forceinline__ int log2_above(double x) { return x > 0.0 ? ilogb(x) + 1 : kZeroExp; }
+// 2^-e as FP64, 0 beyond its normal range (e >= 0)
+__device__ __forceinline__ double exp2_neg64(int e) { return e > 1022 ? 0.0 : __hiloint2double((1023 - e) << 20, 0); }
 
 // InvFFT_1(L^+) of one instance for a block of columns.
 //
@@ -1138,28 +1142,34 @@ __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict
   const int q23 = c2 * c2 + k3 * k3;
   if (threadIdx.x == 0) el = kZeroExp;
   __syncthreads();
+#pragma unroll(N >= 48 ? 1 : 4)
   for (int j = w; j < J; j += WARPS) {
     const size_t u = ((size_t)b * J + j) * N;
     constexpr int R = (N + 31) / 32;  // planes per lane
     int e[R], base = kZeroExp;
-    float f[R];
+    unsigned f[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int i = lane + 32 * r;
       e[r] = i < N ? EP[u + i] : 2 * kZeroExp;
-      f[r] = i < N ? BP[u + i] : 0.f;
+      f[r] = i < N ? __float_as_uint(BP[u + i]) : 0u;
       base = max(base, e[r]);
     }
     base = __reduce_max_sync(0xffffffffu, base);
-    double s = 0.0;
+    // the bounds' 24-bit mantissas at 2^37 (their exponent is 60), added as
+    // integers with 32 bits below: FP64 sums took 3.5 us of the SM's pipe per block at
+    // N = J = 64
+    u64 s = 0;
 #pragma unroll
-    for (int r = 0; r < R; ++r) s += f[r] * exp2_neg(base - e[r]);
+    for (int r = 0; r < R; ++r)
+      if (base - e[r] < 64) s += ((u64)(f[r] & 0x7fffffu | 0x800000u) << 32) >> (base - e[r]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
-      part[j] = s * pm[j];
-      pe[j] = base;
-      atomicMax(&el, base + log2_above(s) - kSumBits - q[j] + 64);
+      s += N;  // past what the shifts dropped
+      part[j] = (double)s * pm[j];
+      pe[j] = base + 5;
+      atomicMax(&el, base + 5 + 64 - __clzll((i64)s) - kSumBits - q[j] + 64);
     }
   }
   __syncthreads();
@@ -1168,7 +1178,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_axis1_acc(const ci64* __restrict
     for (int j = lane + 32; j < J; j += 32) base = max(base, pe[j]);
     base = __reduce_max_sync(0xffffffffu, base);
     double s = 0.0;
-    for (int j = lane; j < J; j += 32) s += scalbn(part[j], pe[j] - base);
+    for (int j = lane; j < J; j += 32) s += part[j] * exp2_neg64(base - pe[j]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {

@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
   store_spectrum<N>(x, t, PW + ((size_t)bj * N + i1) * NC);
   if (tp == 0) {
     EP[(size_t)bj * N + i1] = E;
-    BP[(size_t)bj * N + i1] = plane_bound(top, s);
+    BP[(size_t)bj * N + i1] = plane_bound(top);
   }
 }
 
