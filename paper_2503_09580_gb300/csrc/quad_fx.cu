@@ -100,16 +100,16 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   const double pi = 3.141592653589793238462643383279502884;
   // phi_j carries 4 pi^2 w_j B_j s_j / N^6 (one 1 / N^3 for T+ or T-, one for
   // the last transform); Eq. (2.14): 16 pi^2, and T+ T- a second 1 / N^3
-  const double c0 = 4.0 / ((double)N * N * N);
+  const double c0 = 4.0 / (double)n3, c0_lo = std::fma(-c0, (double)n3, 4.0) / (double)n3;
   int ke = 0;
   const double top = std::frexp(std::sqrt(rule.wmax * c0), &ke);  // top 2^ke, top in [0.5, 1)
   (void)top;
-  const double c = std::scalbn(c0, -2 * ke);
+  const double c = std::scalbn(c0, -2 * ke), c_lo = std::scalbn(c0_lo, -2 * ke);
   int launches = 4;
   auto phases = [&](int c0, int c1) {
     const int m0 = rule.class_begin[c0];
     LBO_LAUNCH(p, "q_fx_phase_table", s, k_q_phase_table<N>, dim3(rule.class_begin[c1] - m0, J), 256, 0, rule.gj, rule.sig,
-               rule.wm, rule.node + m0, c0, c1 - c0, pi, 2.0 * p->L, c, w.tab1, w.tab);
+               rule.wm, rule.node + m0, c0, c1 - c0, pi, 2.0 * p->L, c, c_lo, w.tab1, w.tab);
     launches += 1;
   };
   if (cut.classes == rule.classes) phases(0, rule.classes);
@@ -130,9 +130,9 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   LBO_LAUNCH(p, "q_fx_rescale", s, k_q_rescale<N>, dim3((NC + 63) / 64, B), 64, 0, w.R, w.eR, w.rm, w.EF);
   smem_of(k_q_plane<N>, GeoQ<N>::BYTES);
   smem_of(k_axis1_acc<N, ACC_WARPS>, acc_smem<N, ACC_WARPS>(256));
-  // head room of the sum over m: products of at most 2^60, a sum of at most 2^62
+  // head room of the sum over m: products of at most 2^60, a sum below 2^63
   int guard = 0;
-  while ((4 << guard) < M) ++guard;
+  while ((8 << guard) <= M) ++guard;
   for (int b0 = 0; b0 < B; b0 += cut.G) {
     const int n = std::min(cut.G, B - b0);
     const ci64* R = w.R + b0 * H;

@@ -41,12 +41,21 @@ struct GeoQ {
 // the two images.  With e_1 = c + i s of a class, axis 1 takes
 //   tab1[(j classes + class) N + k1] = ((c + s) s_m, (c - s) s_m), 1 = 2^61,
 // where s_m = sqrt(w_m a): T+ T- then carries w_m and the constant a; the planes
-//   tab[(j nodes + node) NC + (k2, k3)] = e_2(k2) e_3(k3), 1 = 2^62.
+//   tab[(j nodes + node) NC + (k2, k3)] = +- e_2(k2) e_3(k3), 1 = 2^62,
+// negative for every other node: the product T+ T- is the same, and the mean
+// error that the transforms' roundings leave in T+ and T- changes sides.  The
+// large radial nodes, whose T+ and T- hardly meet, weigh it by some hundreds:
+// without this and with ties all rounded up, the mass of Q+ was off by 1 to 5e-15
+// at N = 16 to 32, now by 2e-16 to 2e-15 (FP64 kernels: up to 1e-15).
+// a + a_lo: the constant in two parts.  s_m multiplies every mode of every radial
+// node, so its rounding does not average out: the factors of axis 1 are formed
+// in pairs of FP64 from the FP64 values of c, s and w_m.
 // grid = (nodes, J), block = 256.
 template <int N>
 __global__ void __launch_bounds__(256) k_q_phase_table(const double* __restrict__ gj, const double* __restrict__ sig,
                                                        const double* __restrict__ wm, const int4* __restrict__ node,
                                                        int class0, int classes, double pi, double two_l, double a,
+                                                       double a_lo,
                                                        ci64* __restrict__ tab1, ci64* __restrict__ tab) {
   constexpr int HC = Geo<N>::HC, NC = Geo<N>::NC;
   __shared__ double2 e[2][N];
@@ -61,9 +70,15 @@ __global__ void __launch_bounds__(256) k_q_phase_table(const double* __restrict_
     if (k == N / 2) co = cos(al * (N / 2));
     else sincos(al * (double)centred<N>(k), &s, &co);
     if (d == 0) {
-      const double sm = sqrt(wm[nd.x] * a) * 0x1p61;
-      tab1[((size_t)j * classes + nd.y - class0) * N + k] =
-          ci64{pack_mult(__double2ll_rn((co + s) * sm)), pack_mult(__double2ll_rn((co - s) * sm))};
+      const double w = wm[nd.x], x = __dmul_rn(w, a), xl = fma(w, a, -x) + w * a_lo;
+      const double sm = sqrt(x), sl = (fma(-sm, sm, x) + xl) / (2.0 * sm);
+      auto factor = [&](double b) {  // (co + b) s_m 2^61
+        const double t = __dadd_rn(co, b), u = __dsub_rn(t, co);
+        const double tl = __dadd_rn(__dsub_rn(co, __dsub_rn(t, u)), __dsub_rn(b, u));
+        const double hi = __dmul_rn(t, sm), lo = fma(t, sm, -hi) + (t * sl + tl * sm);
+        return pack_mult(__double2ll_rn(hi * 0x1p61) + __double2ll_rn(lo * 0x1p61));
+      };
+      tab1[((size_t)j * classes + nd.y - class0) * N + k] = ci64{factor(s), factor(-s)};
     } else {
       e[d - 1][k] = double2{co, s};
     }
@@ -72,9 +87,10 @@ __global__ void __launch_bounds__(256) k_q_phase_table(const double* __restrict_
   ci64* out = tab + ((size_t)j * gridDim.x + blockIdx.x) * NC;
   for (int t = threadIdx.x; t < NC; t += 256) {
     const double2 u = e[0][t / HC], v = e[1][t % HC];
-    const i64 s = __double2ll_rn((u.x * v.y + u.y * v.x) * 0x1p62);
+    const double one = blockIdx.x % 2 ? -0x1p62 : 0x1p62;
+    const i64 s = __double2ll_rn((u.x * v.y + u.y * v.x) * one);
     // the planes negate the words of s: its low one is not -2^31
-    out[t] = ci64{pack_mult(__double2ll_rn((u.x * v.x - u.y * v.y) * 0x1p62)),
+    out[t] = ci64{pack_mult(__double2ll_rn((u.x * v.x - u.y * v.y) * one)),
                   pack_mult((unsigned)(u64)s == 0x80000000u ? s + 1 : s)};
   }
 }
@@ -293,7 +309,8 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
       sync();
       if (!G::WARP && threadIdx.x < G::PPC) red[threadIdx.x] = 0;
     } else if (kind == 1) {
-      // T+ and T- of the pencil to at most 2^62, their product, and the sum over m
+      // T+ and T- of the pencil to at most 2^62, their product, and the sum over m;
+      // ties are rounded up and down in turn
       int m = 0;
 #pragma unroll
       for (int i = 0; i < V; ++i) m = max(m, max(abs((int)(x[i].x >> 32)), abs((int)(x[i].y >> 32))));
@@ -305,17 +322,17 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
 #pragma unroll
         for (int i = 0; i < V; ++i) {
           i64& a = acc[idx_halves<N>(i, h) * N + q];
-          a = shift_right(a, d);
+          a = (a + ((i64)1 << (d - 1)) - i % 2) >> d;
         }
         EA = EPr;
       }
       const int d = min(EA - EPr + guard, 62);
-      const i64 half = d > 0 ? (i64)1 << (d - 1) : 0;
+      const i64 half = d > 0 ? (i64)1 << (d - 1) : 0, down = d > 0 ? half - 1 : 0;
 #pragma unroll
       for (int i = 0; i < V; ++i) {
         const SignedMult a = signed_mult((i64)((u64)x[i].y << l));
         const i64 p = mul_signed_rounded((i64)((u64)x[i].x << l), a.m, a.neg);
-        acc[idx_halves<N>(i, h) * N + q] += (p + half) >> d;
+        acc[idx_halves<N>(i, h) * N + q] += (p + (i % 2 ? down : half)) >> d;
       }
     } else if (kind == 2) {
       sync();

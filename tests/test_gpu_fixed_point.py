@@ -243,3 +243,29 @@ def test_cold_thin_gases_whose_outer_planes_vanish(n, theta, rho):
     b = apply(lbo.Plan(n, L, 0.5, n, kernel=1), params, g)
     tol = 2 * 4 * U64 * max(ratio_rms(params, g, n, L)[0], 64.0)
     assert np.abs(a - b).max() <= tol * np.abs(b).max()
+
+
+def quadratic_errors(n, J, p, batch=8):
+    """2-norm errors of Q over a batch of sums of two Maxwellians, as the FP64
+    kernels' and the default's, against pairs of FP64 on the same tables."""
+    L = 8.0
+    rng = np.random.Generator(np.random.PCG64(160 + n))
+    a = workloads.velocity_axis(n, L)
+    f = np.zeros((batch, n, n, n))
+    for b in range(batch):
+        for _ in range(2):
+            rho, th, u = rng.uniform(0.3, 1.0), rng.uniform(0.5, 1.5), rng.uniform(-1.0, 1.0, 3)
+            e = [np.exp(-(a - x) ** 2 / (2 * th)) for x in u]
+            f[b] += rho * (2 * np.pi * th) ** -1.5 * e[0][:, None, None] * e[1][None, :, None] * e[2][None, None, :]
+    out = [apply(lbo.Plan(n, L, 0.5, J, hemisphere_p=p, **kw), np.zeros((batch, 5)), f, quad=True)
+           for kw in ({"precision": "fp64x2"}, {"kernel": 1}, {})]
+    return [np.sqrt(((x - out[0]) ** 2).sum(axis=(1, 2, 3)) / (out[0] ** 2).sum(axis=(1, 2, 3))) for x in out[1:]]
+
+
+@pytest.mark.parametrize("n,J,p", [(16, 16, 4), (16, 9, 2), (16, 9, 4), (32, 17, 4)])
+def test_quadratic_errs_no_more_than_the_fp64_kernels(n, J, p):
+    """Hard spheres weigh the largest radial nodes most, where T+ and T- hardly
+    meet: a mean error of either shows in the mass of Q+.  The errors of a
+    batch, together, stay below those of FP64 transforms."""
+    fp64, fixed = quadratic_errors(n, J, p)
+    assert np.sqrt((fixed ** 2).mean()) <= np.sqrt((fp64 ** 2).mean())
