@@ -128,7 +128,8 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   LBO_LAUNCH(p, "q_fx_axis1_head", s, k_axis1_head<N>, dim3((NC * T + 63) / 64, B, 2), 64, 0, w.F, w.EPh,
              (const ci64*)nullptr, (const int*)nullptr, omega, rule.omega3 ? 1 : 0, omega_exp, 0, w.R, w.eR, w.rm, w.EC, 0);
   LBO_LAUNCH(p, "q_fx_rescale", s, k_q_rescale<N>, dim3((NC + 63) / 64, B), 64, 0, w.R, w.eR, w.rm, w.EF);
-  smem_of(k_q_plane<N>, GeoQ<N>::BYTES);
+  const auto k_plane_m = M < 64 ? k_q_plane<N, false> : k_q_plane<N, true>;
+  smem_of(k_plane_m, GeoQ<N>::BYTES);
   smem_of(k_axis1_acc<N, ACC_WARPS>, acc_smem<N, ACC_WARPS>(256));
   // head room of the sum over m: products of at most 2^60, a sum below 2^63
   int guard = 0;
@@ -143,7 +144,7 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
         if (cut.classes < rule.classes) phases(c0, c1);
         LBO_LAUNCH(p, "q_fx_axis1_phase", s, k_q_axis1<N>, dim3((NC * T + 31) / 32, c1 - c0, np), 32, 0, R, w.tab1, J, q0,
                    w.Z);
-        LBO_LAUNCH(p, "q_fx_plane_prod", s, k_q_plane<N>, dim3(N / GeoQ<N>::PPC, np), GeoQ<N>::THREADS, GeoQ<N>::BYTES,
+        LBO_LAUNCH(p, "q_fx_plane_prod", s, k_plane_m, dim3(N / GeoQ<N>::PPC, np), GeoQ<N>::THREADS, GeoQ<N>::BYTES,
                    w.Z, w.tab, rule.node + m0, c0, c1 - c0, w.EF + b0, J, m1 - m0, q0, c0 == 0 ? 1 : 0,
                    c1 == rule.classes ? 1 : 0, guard, ke, w.accG, w.accE, w.PW, w.EP, w.BP);
         launches += 2;

@@ -198,9 +198,12 @@ __global__ void __launch_bounds__(32) k_q_axis1(const ci64* __restrict__ R, cons
 // instances: 13.9 ms, where the kernel that read a ready Z per node took 10.1
 // and left 7.3 to axis 1.  The exponents of the sum belong to a row, not to the
 // plane: the largest T of a row needs a shuffle, that of a plane a barrier.
+// CARRY, from 64 nodes on: the sum's unit is 2^guard of a product's, and products
+// rounded each by itself would leave more than FP64 transforms do (N = 32, M =
+// 288, hard spheres: up to 3.5 times their error); costs 1 %.
 // EF[b]: exponent of F; 2^ke: factor of the phase table; EP, BP as k_plane's.
 // grid = (N / PPC, pairs), block = GeoQ<N>::THREADS.
-template <int N>
+template <int N, bool CARRY>
 __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(const ci64* __restrict__ Z,
                                                             const ci64* __restrict__ tab, const int4* __restrict__ node,
                                                             int class0, int classes, const int* __restrict__ EF,
@@ -251,6 +254,42 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
   ci64 x[V];
   int E = 0, s = 0;
   float top = 0.f;
+  // the sum += product(i) 2^(EPr - guard), i < V, of the thread's part of a row
+  int carryE = kZeroExp;
+  unsigned carry = 0;
+  auto add = [&](int EPr, auto product) {
+    if (EPr > EA) {  // the sum moves to the larger exponent; ties go up and down in turn
+      const int d = min(EPr - EA, 63);
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        i64& a = acc[idx_halves<N>(i, h) * N + q];
+        a = (a + ((i64)1 << (d - 1)) - i % 2) >> d;
+      }
+      EA = EPr;
+    }
+    const int d = min(EA - EPr + guard, 62);
+    const i64 half = d > 0 ? (i64)1 << (d - 1) : 0;
+    if (CARRY && d < 32) {
+      // what a product loses in the sum's units goes to the row's next point, and
+      // what is left at its end to the next node's
+      unsigned c = (unsigned)half;
+      if (carryE != kZeroExp) c = EPr >= carryE ? carry >> min(EPr - carryE, 31) : carry << (carryE - EPr);
+      const unsigned mask = (1u << d) - 1;
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        const i64 p = product(i) + (i64)c;
+        acc[idx_halves<N>(i, h) * N + q] += p >> d;
+        c = (unsigned)(u64)p & mask;
+      }
+      carry = c;
+      carryE = EPr;
+    } else {
+      const i64 down = d > 0 ? half - 1 : 0;
+#pragma unroll
+      for (int i = 0; i < V; ++i) acc[idx_halves<N>(i, h) * N + q] += (product(i) + (i % 2 ? down : half)) >> d;
+      carryE = kZeroExp;
+    }
+  };
   const int passes = 2 * mc + (last ? 2 : 0);
 #pragma unroll 1
   for (int it = 0; it < passes; ++it) {
@@ -309,30 +348,23 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
       sync();
       if (!G::WARP && threadIdx.x < G::PPC) red[threadIdx.x] = 0;
     } else if (kind == 1) {
-      // T+ and T- of the pencil to at most 2^62, their product, and the sum over m;
-      // ties are rounded up and down in turn
+      // T+ and T- of the pencil to at most 2^62, their product, and the sum over m
       int m = 0;
 #pragma unroll
       for (int i = 0; i < V; ++i) m = max(m, max(abs((int)(x[i].x >> 32)), abs((int)(x[i].y >> 32))));
       if (T == 2) m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
       const int l = max(__clz(m) - 2, 0);
       const int EPr = m ? 2 * (E - l) + 64 + guard : kZeroExp;
-      if (EPr > EA) {  // the sum moves to the larger exponent
-        const int d = min(EPr - EA, 63);
-#pragma unroll
-        for (int i = 0; i < V; ++i) {
-          i64& a = acc[idx_halves<N>(i, h) * N + q];
-          a = (a + ((i64)1 << (d - 1)) - i % 2) >> d;
-        }
-        EA = EPr;
-      }
-      const int d = min(EA - EPr + guard, 62);
-      const i64 half = d > 0 ? (i64)1 << (d - 1) : 0, down = d > 0 ? half - 1 : 0;
-#pragma unroll
-      for (int i = 0; i < V; ++i) {
+      auto product = [&](int i) {
         const SignedMult a = signed_mult((i64)((u64)x[i].y << l));
-        const i64 p = mul_signed_rounded((i64)((u64)x[i].x << l), a.m, a.neg);
-        acc[idx_halves<N>(i, h) * N + q] += (p + (i % 2 ? down : half)) >> d;
+        return mul_signed_rounded((i64)((u64)x[i].x << l), a.m, a.neg);
+      };
+      if constexpr (T == 2) {  // all products first: 1 to 3 % faster here, 2 % slower with all values in one thread
+#pragma unroll
+        for (int i = 0; i < V; ++i) x[i].x = product(i);
+        add(EPr, [&](int i) { return x[i].x; });
+      } else {
+        add(EPr, product);
       }
     } else if (kind == 2) {
       sync();

@@ -262,7 +262,7 @@ def quadratic_errors(n, J, p, batch=8):
     return [np.sqrt(((x - out[0]) ** 2).sum(axis=(1, 2, 3)) / (out[0] ** 2).sum(axis=(1, 2, 3))) for x in out[1:]]
 
 
-@pytest.mark.parametrize("n,J,p", [(16, 16, 4), (16, 9, 2), (16, 9, 4), (32, 17, 4)])
+@pytest.mark.parametrize("n,J,p", [(16, 16, 4), (16, 9, 2), (16, 9, 4), (32, 17, 4), (16, 16, 16), (32, 17, 12)])
 def test_quadratic_errs_no_more_than_the_fp64_kernels(n, J, p):
     """Hard spheres weigh the largest radial nodes most, where T+ and T- hardly
     meet: a mean error of either shows in the mass of Q+.  The errors of a
