@@ -21,6 +21,7 @@ namespace {
 constexpr int N = LBO_FX_N;
 constexpr int NC = Geo<N>::NC, T = Geo<N>::T;
 constexpr size_t H = (size_t)N * NC, n3 = (size_t)N * N * N;
+constexpr int kSMs = 152;
 constexpr int ACC_WARPS = 8, PPC = PlanesPPC<N>::v, CPPC = CombinePPC<N>::v;
 
 // How a call is cut: G instances at a time whose J plane spectra PW stay below
@@ -29,6 +30,7 @@ constexpr int ACC_WARPS = 8, PPC = PlanesPPC<N>::v, CPPC = CombinePPC<N>::v;
 // pairs as many as 1 GB of Z holds, spread evenly over the launches.
 struct Cut {
   int G, classes, nodes, most, pairs;  // nodes, most: the most nodes and pairs of a launch
+  int few;  // launches of at most so many pairs store their products first (k_q_plane)
   Cut(int B, int J, const QuadRule& r) {
     const size_t z = 2 * sizeof(ci64) * H, gb = (size_t)1 << 30;
     G = (int)std::min<size_t>(B, std::max<size_t>(1, (gb / 2) / (sizeof(ci64) * H * J)));
@@ -40,6 +42,9 @@ struct Cut {
     most = (int)std::min<size_t>(all, std::max<size_t>(1, gb / (z * classes)));
     const size_t launches = (all + most - 1) / most;
     pairs = (int)((all + launches - 1) / launches);
+    // fewer blocks than SMs, and products of at most 1 GB
+    few = (int)std::min<size_t>((kSMs - 1) / (N / GeoQ<N>::PPC), gb / (sizeof(i64) * n3 * nodes));
+    few = std::min(few, most);
   }
 };
 
@@ -47,9 +52,9 @@ struct Cut {
 // never needs more, so what was captured with a larger one keeps its buffer.
 struct Buffers {
   ci64 *R, *F, *PW, *Z, *tab1, *tab;
-  i64 *accG, *om3;
+  i64 *accG, *om3, *prod;
   float *rm, *BPh, *BP;
-  int *eR, *EF, *EPh, *EC, *bad, *EP, *accE;
+  int *eR, *EF, *EPh, *EC, *bad, *EP, *accE, *prodE;
   size_t bytes;
   Buffers(void* base, size_t B, size_t J, const QuadRule& r, const Cut& c) {
     unsigned char* p = (unsigned char*)base;
@@ -76,6 +81,8 @@ struct Buffers {
     take(bad, B);
     take(EP, c.G * J * N);
     take(accE, rest ? (size_t)c.most * N * N : 0);
+    take(prod, (size_t)c.few * c.nodes * n3);
+    take(prodE, (size_t)c.few * c.nodes * N * N);
     bytes = (size_t)(p - (unsigned char*)base);
   }
 };
@@ -128,8 +135,11 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   LBO_LAUNCH(p, "q_fx_axis1_head", s, k_axis1_head<N>, dim3((NC * T + 63) / 64, B, 2), 64, 0, w.F, w.EPh,
              (const ci64*)nullptr, (const int*)nullptr, omega, rule.omega3 ? 1 : 0, omega_exp, 0, w.R, w.eR, w.rm, w.EC, 0);
   LBO_LAUNCH(p, "q_fx_rescale", s, k_q_rescale<N>, dim3((NC + 63) / 64, B), 64, 0, w.R, w.eR, w.rm, w.EF);
-  const auto k_plane_m = M < 64 ? k_q_plane<N, false> : k_q_plane<N, true>;
-  smem_of(k_plane_m, GeoQ<N>::BYTES);
+  const bool carry = M >= 64;
+  const auto k_whole = carry ? k_q_plane<N, true, WHOLE> : k_q_plane<N, false, WHOLE>;
+  const auto k_sum = carry ? k_q_plane<N, true, SUM> : k_q_plane<N, false, SUM>;
+  const auto k_products = k_q_plane<N, false, PRODUCTS>;
+  for (const auto k : {k_whole, k_sum, k_products}) smem_of(k, GeoQ<N>::BYTES);
   smem_of(k_axis1_acc<N, ACC_WARPS>, acc_smem<N, ACC_WARPS>(256));
   // head room of the sum over m: products of at most 2^60, a sum below 2^63
   int guard = 0;
@@ -144,9 +154,19 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
         if (cut.classes < rule.classes) phases(c0, c1);
         LBO_LAUNCH(p, "q_fx_axis1_phase", s, k_q_axis1<N>, dim3((NC * T + 31) / 32, c1 - c0, np), 32, 0, R, w.tab1, J, q0,
                    w.Z);
-        LBO_LAUNCH(p, "q_fx_plane_prod", s, k_plane_m, dim3(N / GeoQ<N>::PPC, np), GeoQ<N>::THREADS, GeoQ<N>::BYTES,
-                   w.Z, w.tab, rule.node + m0, c0, c1 - c0, w.EF + b0, J, m1 - m0, q0, c0 == 0 ? 1 : 0,
-                   c1 == rule.classes ? 1 : 0, guard, ke, w.accG, w.accE, w.PW, w.EP, w.BP);
+        const int planes = N / GeoQ<N>::PPC, mc = m1 - m0, f0 = c0 == 0 ? 1 : 0, l1 = c1 == rule.classes ? 1 : 0;
+        auto plane = [&](const char* name, decltype(k_whole) k, dim3 grid, int share) {
+          LBO_LAUNCH(p, name, s, k, grid, GeoQ<N>::THREADS, GeoQ<N>::BYTES, w.Z, w.tab, rule.node + m0, c0, c1 - c0,
+                     w.EF + b0, J, mc, q0, f0, l1, guard, ke, share, w.prod, w.prodE, w.accG, w.accE, w.PW, w.EP, w.BP);
+        };
+        if (np > cut.few) {
+          plane("q_fx_plane_prod", k_whole, dim3(planes, np), 0);
+        } else {  // one wave of blocks
+          const int wave = kSMs * std::max(GeoQ<N>::BLOCKS, 2), share = (mc * planes * np + wave - 1) / wave;
+          plane("q_fx_plane_prod", k_products, dim3(planes, np, (mc + share - 1) / share), share);
+          plane("q_fx_plane_sum", k_sum, dim3(planes, np), 0);
+          launches += 1;
+        }
         launches += 2;
       }
     }

@@ -201,13 +201,20 @@ __global__ void __launch_bounds__(32) k_q_axis1(const ci64* __restrict__ R, cons
 // CARRY, from 64 nodes on: the sum's unit is 2^guard of a product's, and products
 // rounded each by itself would leave more than FP64 transforms do (N = 32, M =
 // 288, hard spheres: up to 3.5 times their error); costs 1 %.
+// A launch with few pairs would leave SMs idle while its blocks walk the nodes
+// one after the other.  PRODUCTS takes `share` of them per block and stores
+// the products (prod, prodE: [pair][node][i1]) that SUM then adds in the same
+// order: the same bits.  N = 16, one instance, one radial node, M = 32: 206 us as
+// a whole, 87 in two (153 in FP64 registers or shared memory).
 // EF[b]: exponent of F; 2^ke: factor of the phase table; EP, BP as k_plane's.
-// grid = (N / PPC, pairs), block = GeoQ<N>::THREADS.
-template <int N, bool CARRY>
+// grid = (N / PPC, pairs), for PRODUCTS (N / PPC, pairs, ceil(mc / share)), block = GeoQ<N>::THREADS.
+enum QMode { WHOLE, PRODUCTS, SUM };
+template <int N, bool CARRY, int MODE>
 __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(const ci64* __restrict__ Z,
                                                             const ci64* __restrict__ tab, const int4* __restrict__ node,
                                                             int class0, int classes, const int* __restrict__ EF,
                                                             int J, int mc, int bj0, int first, int last, int guard, int ke,
+                                                            int share, i64* __restrict__ prod, int* __restrict__ prodE,
                                                             i64* __restrict__ accG, int* __restrict__ accE,
                                                             ci64* __restrict__ PW, int* __restrict__ EP,
                                                             float* __restrict__ BP) {
@@ -241,7 +248,7 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
   if (first) {
 #pragma unroll
     for (int i = 0; i < V; ++i) acc[idx_halves<N>(i, h) * N + q] = 0;
-  } else {
+  } else if (MODE != PRODUCTS) {
 #pragma unroll
     for (int i = 0; i < V; ++i) acc[idx_halves<N>(i, h) * N + q] = accG[pl * N * N + idx_halves<N>(i, h) * N + q];
     EA = accE[pl * N + q];
@@ -290,11 +297,21 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
       carryE = kZeroExp;
     }
   };
-  const int passes = 2 * mc + (last ? 2 : 0);
+  if (MODE == SUM) {
 #pragma unroll 1
-  for (int it = 0; it < passes; ++it) {
+    for (int m = 0; m < mc; ++m) {
+      const size_t pm = ((size_t)blockIdx.y * mc + m) * N + i1;
+#pragma unroll
+      for (int i = 0; i < V; ++i) x[i].x = prod[pm * N * N + idx_halves<N>(i, h) * N + q];
+      add(prodE[pm * N + q], [&](int i) { return x[i].x; });
+    }
+  }
+  const int begin = MODE == PRODUCTS ? 2 * share * (int)blockIdx.z : (MODE == SUM ? 2 * mc : 0);
+  const int passes = MODE == PRODUCTS ? min(begin + 2 * share, 2 * mc) : 2 * mc + (last ? 2 : 0);
+#pragma unroll 1
+  for (int it = begin; it < passes; ++it) {
     const int kind = it >= 2 * mc ? 2 + (it - 2 * mc) : it & 1;
-    if (kind == 0) {
+    if (MODE != SUM && kind == 0) {
       // Z(k2, q) = c Z1 + s Z2, e_2 e_3 = c + i s.  Beyond the half spectrum,
       // from its mirrored entry: the parts of c Z2 - s Z1, exchanged.
       const int4 nd = node[it >> 1];
@@ -314,10 +331,10 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
         x[i] = ci64{mir ? zy : zx, mir ? zx : zy};
       }
       E = E0;
-    } else if (kind == 1) {
+    } else if (MODE != SUM && kind == 1) {
 #pragma unroll
       for (int i = 0; i < V; ++i) x[i] = Bs[q * RS + idx_parity<N>(i, h)];
-    } else if (kind == 2) {
+    } else if (MODE != PRODUCTS && kind == 2) {
       // the rows to one exponent; rows q and q + N/2 of the sum, parts exchanged
       const int top = (int)group_max((unsigned)(EA - 2 * kZeroExp), 4) + 2 * kZeroExp, d = min(top - EA, 63);
 #pragma unroll
@@ -333,21 +350,21 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
         x[i] = fwd ? ci64{a[q + N / 2], a[q]} : ci64{0, 0};
       }
       E = EA == kZeroExp ? 0 : EA;
-    } else if (fwd) {
+    } else if (MODE != PRODUCTS && fwd) {
       load_columns<N>(x, t, Bs);
     }
     top = __uint_as_float(group_max(__float_as_uint(pencil_sum<N>(abs_sum<V>(x))), kind));
     s = shift_for(top, kSumBits);
     shift_all<V>(x, s);
     E += s;
-    pencil_inverse<N>(x, h, kind < 2);
-    if (kind == 0) {
+    pencil_inverse<N>(x, h, MODE == PRODUCTS || (MODE == WHOLE && kind < 2));
+    if (MODE != SUM && kind == 0) {
 #pragma unroll
       for (int i = 0; i < V; ++i) Bs[idx_halves<N>(i, h) * RS + q] = x[i];
       if (!G::WARP && threadIdx.x < G::PPC) red[G::PPC + threadIdx.x] = 0;
       sync();
       if (!G::WARP && threadIdx.x < G::PPC) red[threadIdx.x] = 0;
-    } else if (kind == 1) {
+    } else if (MODE != SUM && kind == 1) {
       // T+ and T- of the pencil to at most 2^62, their product, and the sum over m
       int m = 0;
 #pragma unroll
@@ -359,19 +376,27 @@ __global__ void __launch_bounds__(GeoQ<N>::THREADS, GeoQ<N>::BLOCKS) k_q_plane(c
         const SignedMult a = signed_mult((i64)((u64)x[i].y << l));
         return mul_signed_rounded((i64)((u64)x[i].x << l), a.m, a.neg);
       };
-      if constexpr (T == 2) {  // all products first: 1 to 3 % faster here, 2 % slower with all values in one thread
+      if (MODE == PRODUCTS) {
+        const size_t pm = ((size_t)blockIdx.y * mc + (it >> 1)) * N + i1;
 #pragma unroll
-        for (int i = 0; i < V; ++i) x[i].x = product(i);
-        add(EPr, [&](int i) { return x[i].x; });
+        for (int i = 0; i < V; ++i) prod[pm * N * N + idx_halves<N>(i, h) * N + q] = product(i);
+        if (h == 0) prodE[pm * N + q] = EPr;
       } else {
-        add(EPr, product);
+        if constexpr (T == 2) {  // all products first: 1 to 3 % faster here, 2 % slower with all values in one thread
+#pragma unroll
+          for (int i = 0; i < V; ++i) x[i].x = product(i);
+          add(EPr, [&](int i) { return x[i].x; });
+        } else {
+          add(EPr, product);
+        }
       }
-    } else if (kind == 2) {
+    } else if (MODE != PRODUCTS && kind == 2) {
       sync();
       if (fwd) store_rows<N>(x, t, Bs);
       sync();
     }
   }
+  if (MODE == PRODUCTS) return;
   if (!last) {
 #pragma unroll
     for (int i = 0; i < V; ++i) accG[pl * N * N + idx_halves<N>(i, h) * N + q] = acc[idx_halves<N>(i, h) * N + q];

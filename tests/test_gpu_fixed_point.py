@@ -269,3 +269,22 @@ def test_quadratic_errs_no_more_than_the_fp64_kernels(n, J, p):
     batch, together, stay below those of FP64 transforms."""
     fp64, fixed = quadratic_errors(n, J, p)
     assert np.sqrt((fixed ** 2).mean()) <= np.sqrt((fp64 ** 2).mean())
+
+
+@pytest.mark.parametrize("n,J,p,batch,kw", [(16, 1, 4, 40, {}), (16, 3, 8, 17, {}), (24, 2, 1, 29, {}), (24, 5, 6, 11, {}),
+                                            (32, 1, 3, 9, {}), (32, 2, 6, 5, {}), (48, 1, 2, 5, {}),
+                                            (64, 1, 2, 4, {"q_sinc_quadrature": 1}), (64, 2, 6, 2, {})])
+def test_quadratic_of_few_instances_is_that_of_a_batch(n, J, p, batch, kw):
+    """A launch with fewer blocks than SMs stores the products of the hemisphere
+    nodes and adds them in a second kernel, in the order and with the bits of
+    the launch that a batch takes; the first and the last instance, whose share
+    of nodes per block differ with the batch."""
+    L = 8.0
+    _, g = workloads.batched_instances(n, L, batch=batch, seed=170 + n, noise=0.0)
+    params = np.zeros((batch, 5))
+    plan = lbo.Plan(n, L, 0.5, J, hemisphere_p=p, **kw)
+    whole = apply(plan, params, g, quad=True)
+    for i in (0, batch - 1):
+        assert np.array_equal(apply(plan, params[i:i + 1], g[i:i + 1], quad=True)[0], whole[i])
+    two = apply(plan, params[:2], g[:2], quad=True)
+    assert np.array_equal(two, whole[:2])
