@@ -30,7 +30,7 @@ struct Buffers {
   ci64 *R, *F, *MH;  // r^; fields L+, u, w (first: FFT(r), FFT(g) of the planes); M's factors
   i64* mh;
   double* inst;
-  float *rm, *ub, *BPh;
+  float *rm, *ub;
   int *eR, *em, *eM, *EPh, *EC, *bad;
   // of G instances
   ci64* W;
@@ -49,7 +49,6 @@ struct Buffers {
     take(MH, B * 3 * N);
     take(mh, B * n3);
     take(inst, B * Inst<N>::SIZE);
-    take(BPh, 2 * B * N);
     take(rm, B * BANDS * NC);
     take(eR, B * NC);
     take(em, B * N);
@@ -183,7 +182,7 @@ lbo_status LBO_CAT(apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const double
   // r^ = FFT(r); InvFFT_1 of g^ omega and of M^ omega
   smem_of(k_fwd_planes<N, PPC>, Planes<N, PPC>::BYTES);
   LBO_LAUNCH(p, "fx_plane_fwd", s, (k_fwd_planes<N, PPC>), dim3(N / PPC, B, 2), (Planes<N, PPC>::THREADS),
-             (Planes<N, PPC>::BYTES), g, inst, 1, p->cutoff, w.F, w.EPh, w.BPh, w.bad);
+             (Planes<N, PPC>::BYTES), g, inst, 1, p->cutoff, w.F, w.EPh, w.bad);
   launch_head(p, tb, w, B, 0, mc ? 2 : 3, "fx_axis1_head");
   int launches = have ? 3 : 5;
   static_assert(acc_smem<N, ACC_WARPS>(256) <= 226 * 1024, "shared memory of k_axis1_acc at the most radial nodes");

@@ -884,7 +884,7 @@ __device__ __forceinline__ unsigned plane_umax(unsigned v, unsigned* slot) {
   }
 }
 // Axes 3 and 2 of FFT(r) (blockIdx.z = 0 with with_ratio; r = g/M with the
-// cut-off) or of FFT(g): F[z][b][i1][k2][k3], EP and BP [z][b][i1].  The field's plane is
+// cut-off) or of FFT(g): F[z][b][i1][k2][k3], EP [z][b][i1].  The field's plane is
 // read coalesced into shared memory as FP64, converted at the plane's own
 // exponent by the row threads.  Latency-bound: 0.19 ms for 256 instances at N =
 // 32 (1.4 in FP64).
@@ -893,7 +893,7 @@ template <int N, int PPC>
 __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const double* __restrict__ field,
                                                                       const double* __restrict__ inst, int with_ratio, int cutoff,
                                                                       ci64* __restrict__ F, int* __restrict__ EP,
-                                                                      float* __restrict__ BP, int* __restrict__ bad) {
+                                                                      int* __restrict__ bad) {
   constexpr int NC = Geo<N>::NC, V = Geo<N>::V, TPP = Geo<N>::TPP, RS = N + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned red[3 * PPC];
@@ -934,7 +934,6 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
   if (!fin && t.tp == 0) atomicOr(bad + b, 1);
   int E = (int)(top >> 20) - 1023 - 57;  // the plane's largest value in [2^57, 2^58)
   int s = 0;
-  float sum = 0.f;
   ci64 x[V];
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
@@ -947,7 +946,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
     } else {
       load_columns<N>(x, t, Bs);
     }
-    sum = normalise<N>(x, s, E, red + (1 + pass) * PPC + t.pp, true);
+    normalise<N>(x, s, E, red + (1 + pass) * PPC + t.pp, true);
     pencil_inverse<N>(x, t.h, false);
     if (pass == 0) {
       plane_sync<N>();  // D has been read
@@ -957,10 +956,7 @@ __global__ void __launch_bounds__(Planes<N, PPC>::THREADS) k_fwd_planes(const do
   }
   E -= 1;
   store_spectrum<N>(x, t, F + (u * N + i1) * NC);
-  if (t.tp == 0) {
-    EP[u * N + i1] = E;
-    BP[u * N + i1] = plane_bound(sum);
-  }
+  if (t.tp == 0) EP[u * N + i1] = E;
 }
 
 // a value as a multiplier with its sign mask

@@ -53,7 +53,7 @@ struct Cut {
 struct Buffers {
   ci64 *R, *F, *PW, *Z, *tab1, *tab;
   i64 *accG, *om3, *prod;
-  float *rm, *BPh, *BP;
+  float *rm, *BP;
   int *eR, *EF, *EPh, *EC, *bad, *EP, *accE, *prodE;
   size_t bytes;
   Buffers(void* base, size_t B, size_t J, const QuadRule& r, const Cut& c) {
@@ -71,7 +71,6 @@ struct Buffers {
     take(tab, J * c.nodes * NC);
     take(accG, rest ? c.most * n3 : 0);
     take(om3, r.omega3 ? H : 0);
-    take(BPh, B * N);
     take(BP, c.G * J * N);
     take(rm, B * BANDS * NC);
     take(eR, B * NC);
@@ -131,7 +130,7 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   // F = FFT(f); InvFFT_1(F omega)
   smem_of(k_fwd_planes<N, PPC>, Planes<N, PPC>::BYTES);
   LBO_LAUNCH(p, "q_fx_plane_fwd", s, (k_fwd_planes<N, PPC>), dim3(N / PPC, B, 1), (Planes<N, PPC>::THREADS),
-             (Planes<N, PPC>::BYTES), f, (const double*)nullptr, 0, 0, w.F, w.EPh, w.BPh, w.bad);
+             (Planes<N, PPC>::BYTES), f, (const double*)nullptr, 0, 0, w.F, w.EPh, w.bad);
   LBO_LAUNCH(p, "q_fx_axis1_head", s, k_axis1_head<N>, dim3((NC * T + 63) / 64, B, 2), 64, 0, w.F, w.EPh,
              (const ci64*)nullptr, (const int*)nullptr, omega, rule.omega3 ? 1 : 0, omega_exp, 0, w.R, w.eR, w.rm, w.EC, 0);
   LBO_LAUNCH(p, "q_fx_rescale", s, k_q_rescale<N>, dim3((NC + 63) / 64, B), 64, 0, w.R, w.eR, w.rm, w.EF);
