@@ -57,18 +57,23 @@ typedef enum {
 typedef enum {
   LBO_PREC_FP64 = 0,     /* the FP64 path.  Default kernels: FP64 inputs,
                             Maxwellians, ratio and combination, transforms
-                            and products of numbers with 64 bits and a common
-                            exponent per block (at least as accurate as FP64
-                            transforms); LBO_OPT_KERNEL 1 and 2: FP64
-                            throughout                                      */
+                            and products of 64-bit integers with a common
+                            exponent per block: rounded at 2^-57 or less of
+                            a block's largest number, so a number far below
+                            it has fewer digits than FP64's 53.  2-norm error
+                            over batches: 0.1 to 0.6 of the FP64 kernels' in
+                            L, 0.4 to 0.9 in Q; single noise-free instances
+                            up to 3 times (below 4e-14).  LBO_OPT_KERNEL 1
+                            and 2: FP64 throughout                          */
   LBO_PREC_FP32 = 1,     /* FP32 transforms and products, FP64 in/out,
                             FP64 Maxwellians, cut-off and final combination */
-  LBO_PREC_FP32X2 = 2,   /* at least 48 significant bits in transforms and
-                            products; FP64 Maxwellians, ratio, cut-off and
-                            combination.  Default kernels: those of FP64
-                            (faster here and more accurate); LBO_OPT_KERNEL 1:
-                            pairs of FP32 numbers (hi + lo, FP32 exponent
-                            range) on the FP32 pipe                         */
+  LBO_PREC_FP32X2 = 2,   /* errors of a 48-bit arithmetic or less in
+                            transforms and products; FP64 Maxwellians, ratio,
+                            cut-off and combination.  Default kernels: those
+                            of FP64 (faster and more accurate than pairs; Q
+                            of one radial node and one instance up to 20 %
+                            slower); LBO_OPT_KERNEL 1: pairs of FP32 numbers
+                            (hi + lo, FP32 exponent range) on the FP32 pipe */
   LBO_PREC_FP64X2 = 3,   /* transforms and products in pairs of FP64 numbers
                             (about 106 significant bits): the higher-
                             precision convolution of Sec. 3.4 (the paper
@@ -95,8 +100,10 @@ typedef enum {
                               momentum and energy (least squares on the grid) */
   LBO_OPT_HEMISPHERE_P = 6,/* hemisphere rule order p: M = 2 p^2 points (4)   */
   LBO_OPT_PRECISION = 7,   /* lbo_precision                                   */
-  LBO_OPT_KERNEL = 8,      /* 0: fastest built kernel set for (N, precision)
-                              (default; FP64: fixed point on the integer pipe),
+  LBO_OPT_KERNEL = 8,      /* 0 (default): the fastest kernel set built in the
+                              plan's precision (FP64, FP32X2: fixed point on the
+                              integer pipe; FP32: fused at N = 32, generic at
+                              the other N, where the FP64 default is faster),
                               1: the generic plane/axis kernels (FP64 at N = 32
                               runs the hot ones of L and of Q(f,f) with one
                               thread per pencil in registers), 2: the generic
@@ -109,12 +116,22 @@ typedef enum {
                               its hemisphere quadrature
                               sum_m w_m cos(pi g_j sigma_m . k / L), the
                               second mass fix of Sec. 2.3 (Eq. (2.16)): Q^_0
-                              vanishes up to rounding.  Takes the generic
-                              kernels (also for FP32 at N = 32); 0: off   */
+                              vanishes up to rounding.  FP32 then takes the
+                              generic kernels at N = 32 too; 0: off       */
   LBO_OPT_PLANES = 11      /* planes per CTA of the FP64 plane kernel of the gain
                               loop at N = 32 (2, 4 or 8; 0: default, 4): the
                               tile shape lbo_plan_autotune picks for FP64   */
 } lbo_option;
+
+/* Device memory of a plan's default FP64 and FP32X2 kernels, kept between calls
+ * and grown by need: L[g] per instance 6 half spectra of 16 bytes (2 GB at
+ * most, then in parts), and per instance of a group J half spectra and octants
+ * of u^_j (together about 1.3 GB at most, one instance at least: 11 MB at
+ * N = J = 32, 170 MB at 64); a cached call reserves the same.  The Maxwellian
+ * cache: 8 bytes per octant point and radial node, 16 per grid point, per
+ * instance.  Q(f,f): up to 3 half spectra per instance (2 GB), 0.5 GB of plane
+ * spectra, 1 GB each of axis-1 spectra, phase factors and, for few instances,
+ * products.  A smaller batch never needs more than a larger one. */
 
 /* Create a plan for N^3 grids on [-box, box]^3, VHS exponent vhs_omega in
  * [0.5, 1], radial_nodes Gauss-Legendre nodes on [0, R] (Eq. (2.13)).

@@ -136,7 +136,7 @@ void lbo_group_destroy(lbo_group* G) {
   delete G;
 }
 
-// Planes per CTA of the FP64 register plane kernel (N = 32): 2, 4 or 8,
+// Planes per CTA of the FP64 plane kernel of the gain loop (N = 32): 2, 4 or 8,
 // each timed over three applications after one untimed.
 static lbo_status autotune_planes(lbo_plan* p, const double* params, const double* g, double* out, int batch,
                                   int* choice) {
@@ -146,10 +146,10 @@ static lbo_status autotune_planes(lbo_plan* p, const double* params, const doubl
   cudaEventCreate(&b);
   float best = 1e30f;
   int best_p = 0;
-  const int keep = p->r64_planes;
+  const int keep = p->planes_per_cta;
   lbo_status st = LBO_OK;
   for (int P : cands) {
-    p->r64_planes = P;
+    p->planes_per_cta = P;
     st = lbo_apply_linearized(p, params, g, out, batch);
     if (st != LBO_OK) break;
     cudaEventRecord(a, p->stream);
@@ -165,8 +165,8 @@ static lbo_status autotune_planes(lbo_plan* p, const double* params, const doubl
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  p->r64_planes = st == LBO_OK ? best_p : keep;
-  if (choice) *choice = p->r64_planes;
+  p->planes_per_cta = st == LBO_OK ? best_p : keep;
+  if (choice) *choice = p->planes_per_cta;
   return st;
 }
 

@@ -202,8 +202,8 @@ lbo_status LBO_CAT(apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const double
     }
     LBO_LAUNCH(p, "fx_unit_scale", s, k_unit_scale<N>, dim3(J, n), 256, 0, ub, eU, w.rm + b0 * (size_t)BANDS * NC, eR, w.EA, J);
     LBO_LAUNCH(p, "fx_axis1_uhat_inv", s, k_axis1_inv<N>, dim3((NC * T + 63) / 64, J, n), 64, 0, R, eR, U, eU, w.EA, w.W);
-    if (N == 32 && p->r64_planes == 2) launch_planes<N == 32 ? 2 : PPC>(p, w, mh + b0 * n3, em + b0 * N, n);
-    else if (N == 32 && p->r64_planes == 8) launch_planes<N == 32 ? 8 : PPC>(p, w, mh + b0 * n3, em + b0 * N, n);
+    if (N == 32 && p->planes_per_cta == 2) launch_planes<N == 32 ? 2 : PPC>(p, w, mh + b0 * n3, em + b0 * N, n);
+    else if (N == 32 && p->planes_per_cta == 8) launch_planes<N == 32 ? 8 : PPC>(p, w, mh + b0 * n3, em + b0 * N, n);
     else launch_planes<PPC>(p, w, mh + b0 * n3, em + b0 * N, n);
     LBO_LAUNCH(p, "fx_axis1_fwd_acc", s, (k_axis1_acc<N, ACC_WARPS>), dim3((NC * T + 31) / 32, n), 32 * ACC_WARPS,
                smem, w.W, w.EP, w.BP, tb.phi, tb.phi_exp, tb.phi_max, w.F + b0 * H, w.EC + b0 * (size_t)NC, J);

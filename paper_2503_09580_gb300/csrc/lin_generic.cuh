@@ -135,8 +135,8 @@ static lbo_status run_linearized_generic(lbo_plan* p, const GenericTables<T>& tb
           LBO_LAUNCH(p, "plane_inv_mh_fwd", s, k, dim3(N / RP, B), r64::PlaneR<RP>::THREADS, r64::PlaneR<RP>::BYTES,
                      (const double*)R2, W1);
         };
-        if (p->r64_planes == 2) go(std::integral_constant<int, 2>());
-        else if (p->r64_planes == 8) go(std::integral_constant<int, 8>());
+        if (p->planes_per_cta == 2) go(std::integral_constant<int, 2>());
+        else if (p->planes_per_cta == 8) go(std::integral_constant<int, 8>());
         else go(std::integral_constant<int, 4>());
         return;
       }

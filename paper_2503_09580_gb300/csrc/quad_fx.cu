@@ -106,16 +106,15 @@ lbo_status LBO_CAT(q_apply_, LBO_FX_N)(lbo_plan* p, const Tables& tb, const Quad
   const double pi = 3.141592653589793238462643383279502884;
   // phi_j carries 4 pi^2 w_j B_j s_j / N^6 (one 1 / N^3 for T+ or T-, one for
   // the last transform); Eq. (2.14): 16 pi^2, and T+ T- a second 1 / N^3
-  const double c0 = 4.0 / (double)n3, c0_lo = std::fma(-c0, (double)n3, 4.0) / (double)n3;
+  const double a0 = 4.0 / (double)n3, a0_lo = std::fma(-a0, (double)n3, 4.0) / (double)n3;
   int ke = 0;
-  const double top = std::frexp(std::sqrt(rule.wmax * c0), &ke);  // top 2^ke, top in [0.5, 1)
-  (void)top;
-  const double c = std::scalbn(c0, -2 * ke), c_lo = std::scalbn(c0_lo, -2 * ke);
+  std::frexp(std::sqrt(rule.wmax * a0), &ke);  // the largest s_m is 2^ke times a number in [0.5, 1)
+  const double a = std::scalbn(a0, -2 * ke), a_lo = std::scalbn(a0_lo, -2 * ke);
   int launches = 4;
-  auto phases = [&](int c0, int c1) {
-    const int m0 = rule.class_begin[c0];
-    LBO_LAUNCH(p, "q_fx_phase_table", s, k_q_phase_table<N>, dim3(rule.class_begin[c1] - m0, J), 256, 0, rule.gj, rule.sig,
-               rule.wm, rule.node + m0, c0, c1 - c0, pi, 2.0 * p->L, c, c_lo, w.tab1, w.tab);
+  auto phases = [&](int first, int last) {  // classes [first, last)
+    const int m0 = rule.class_begin[first];
+    LBO_LAUNCH(p, "q_fx_phase_table", s, k_q_phase_table<N>, dim3(rule.class_begin[last] - m0, J), 256, 0, rule.gj, rule.sig,
+               rule.wm, rule.node + m0, first, last - first, pi, 2.0 * p->L, a, a_lo, w.tab1, w.tab);
     launches += 1;
   };
   if (cut.classes == rule.classes) phases(0, rule.classes);
