@@ -6,12 +6,13 @@ g = M * (quartic polynomial, N(0,1) coefficients) + 1e-3 N(0,1) grid noise.
 
 One step = one lbo_apply_linearized call over the whole batch (every kernel
 of the path).  The headline value is the FP64 path (FP64 data and
-Maxwellians, transforms in 64-bit fixed point that err no more than FP64
-ones); the same path with FP64 transforms throughout, the FP32 form, the VHS exponents 0.5 / 0.74 / 1.0 and the
-solver and N = 64 workloads are reported beside it, each precision form
-with its measured error against the oracle and its stated bound.  The ALU
-peaks of the roofline fractions are measured in the run
-(lbo_measure_alu_peaks); the HBM peak is the machine's measured copy bandwidth.
+Maxwellians, transforms in 64-bit fixed point, rounded at 2^-57 of a block's
+largest number; the error is reported beside the value); the same path with
+FP64 transforms throughout, the FP32 form, the VHS exponents 0.5 / 0.74 / 1.0
+and the solver and N = 64 workloads are reported too, each precision form
+with its measured error against the oracle and its stated bound.  The peaks
+of the roofline fractions are measured in the run (lbo_measure_alu_peaks,
+lbo_measure_fx_peak); the HBM peak is the machine's measured copy bandwidth.
 Prints one JSON line (rank 0): the headline with its configuration, peaks,
 errors and clocks, below 3 KB.  The whole record, with every kernel, variant and
 workload, goes to stderr as one line, and to a file with --details.
@@ -55,11 +56,6 @@ BOUND_FACTOR = 4.0
 HBM_FALLBACK_GBS = 6800.0
 # Kernels bound by memory traffic, not by their arithmetic (rated in GB/s).
 HBM_KERNELS = ("combine", "conservation_fix", "f32_head", "f32_tail", "tc_combine", "mh_table", "fx_mh_table")
-# Fixed-point transforms (fx64.cuh) run on the integer pipe.  Their peak: a
-# 32-point complex transform held in registers, nothing else running, takes 22
-# SM clocks per transform (measured on a GB300, all warps busy): 2.5 * 2 * 32 *
-# log2(32) = 800 conventional flops, 36.4 per SM and clock.
-FX_FLOPS_PER_SM_CLOCK = 800.0 / 22.0
 # DRAM bytes (read + write) per launch of a dominant kernel at the benchmark
 # workload from one ncu capture, with the sha256 (first 16 hex digits) of the
 # source files it was built from; reported as null once those sources change.
@@ -202,8 +198,9 @@ def tensor_peak():
 
 
 def fx_peak_tflops(peaks):
-    """Rate of the fixed-point register transforms on the integer pipe."""
-    return FX_FLOPS_PER_SM_CLOCK * peaks["sm_count"] * peaks["sm_mhz"] * 1e6 / 1e12
+    """Rate of the fixed-point transforms (fx64.cuh) in registers on the integer
+    pipe, measured in the run (lbo_measure_fx_peak)."""
+    return peaks["fx_tflops"]
 
 
 def instances_per_launch(prof, name, batch):
@@ -513,9 +510,8 @@ def dominant_roofline(prof, precision, peaks, hbm, hbm_src, groups=1):
                              % ("DFMA" if precision == "fp64" else "FFMA", peaks["sm_count"], peaks["sm_mhz"])}
         if name in FX_KERNELS:
             rf.update({"bound": "integer alu", "peak": fx_peak_tflops(peaks), "frac_of_fp64_peak": ach / peaks["fp64_tflops"],
-                       "peak_source": "64-bit fixed-point 32-point transforms in registers, %.1f conventional flops per "
-                                      "SM and clock measured, %d SMs at %.0f MHz of this run"
-                                      % (FX_FLOPS_PER_SM_CLOCK, peaks["sm_count"], peaks["sm_mhz"])})
+                       "peak_source": "measured in this run (lbo_measure_fx_peak: 64-bit fixed-point 32-point transforms "
+                                      "in registers)"})
     rf.update({"frac": rf["achieved"] / rf["peak"], "traffic": ncu_traffic(name, N_GRID, precision),
                "kernel": name, "kernel_share": share, "kernel_ms_per_launch": per,
                "apply_flops_per_instance": apply_flops_per_instance(N_GRID, N_GRID)})
@@ -1138,7 +1134,7 @@ def run_ours(args, world, rank, local):
     params, g = workloads.batched_instances(N_GRID, BOX, batch=BATCH, seed=args.seed + rank, noise=1e-3)
     tp, tg = torch.from_numpy(params).to(dev), torch.from_numpy(g).to(dev)
     stream = torch.cuda.current_stream(dev)
-    peaks = lbo.measure_alu_peaks(stream)
+    peaks = dict(lbo.measure_alu_peaks(stream), fx_tflops=lbo.measure_fx_peak(stream))
     hbm, hbm_src = hbm_peak()
     plan = lbo.Plan(N_GRID, BOX, args.omega, N_GRID, precision=prec)
     if args.eps is not None:
@@ -1323,7 +1319,7 @@ def main():
     if args.q_only:
         import torch
         from paper_2503_09580_gb300 import lbo
-        peaks = lbo.measure_alu_peaks(torch.cuda.current_stream())
+        peaks = dict(lbo.measure_alu_peaks(), fx_tflops=lbo.measure_fx_peak())
         print(json.dumps({"quadratic": {"fp64": quadratic_leg("fp64", peaks), "fp32": quadratic_leg("fp32", peaks)},
                           "measured_peaks": peaks}), flush=True)
         return

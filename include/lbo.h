@@ -586,6 +586,13 @@ lbo_status lbo_vec_combination(lbo_plan *plan, double *y, const double *V, size_
 lbo_status lbo_measure_alu_peaks(void *stream, double *fp32_tflops, double *fp64_tflops, int *sm_count,
                                  double *sm_mhz);
 
+/* The same for the fixed-point transforms of the FP64 default: 32-point
+ * complex transforms of 64-bit integers held in registers, nothing else
+ * running, in TFLOP/s of their conventional 5 N log2 N flops (about 11 on a
+ * GB300, where FP64 FMAs reach 1.26).  Best of three launches; synchronizes
+ * `stream`.  Errors: LBO_ECUDA, LBO_ENOMEM. */
+lbo_status lbo_measure_fx_peak(void *stream, double *tflops);
+
 /* Free a plan (NULL is allowed). */
 void lbo_plan_destroy(lbo_plan *plan);
 

@@ -23,6 +23,7 @@
 
 #include <algorithm>
 
+#include "fx64.cuh"
 #include "lbo_internal.h"
 
 namespace lbo {
@@ -57,6 +58,26 @@ __global__ void __launch_bounds__(kThreads) k_fma_chains(T* sink, long long* cyc
     const long long c1 = clock64();
     if (threadIdx.x == 0) atomicMax((unsigned long long*)cycles, (unsigned long long)(c1 - c0));
   }
+}
+
+// 32-point fixed-point transforms (fx64.cuh) of values that stay in registers,
+// one per thread, four (32^2 times the identity) to a shift back: what the
+// integer pipe makes of the transforms when nothing else runs.
+constexpr int kFxThreads = 64, kFxBlocksPerSM = 4;
+__global__ void __launch_bounds__(kFxThreads) k_fx_transforms(long long* sink, int iters) {
+  fx::ci64 x[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) x[i] = fx::ci64{(long long)(threadIdx.x + i) << 24, (long long)(blockIdx.x - 3 * i) << 20};
+  for (int it = 0; it < iters; ++it) {
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) fx::dft<32, false>(x);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i] = fx::ci64{x[i].x >> 10, x[i].y >> 10};
+  }
+  long long s = 0;
+#pragma unroll
+  for (int i = 0; i < 32; ++i) s ^= x[i].x + x[i].y;
+  sink[blockIdx.x * kFxThreads + threadIdx.x] = s;
 }
 
 // Best rate (TFLOP/s) of k_fma_chains<T, ACC, CLK> over three launches; with
@@ -127,5 +148,42 @@ extern "C" lbo_status lbo_measure_alu_peaks(void* stream, double* fp32_tflops, d
   if (fp64_tflops) *fp64_tflops = f64;
   if (sm_count) *sm_count = sms;
   if (sm_mhz) *sm_mhz = std::max(mhz32, mhz64);
+  return LBO_OK;
+}
+
+extern "C" lbo_status lbo_measure_fx_peak(void* stream, double* tflops) {
+  constexpr int kIters = 1000;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return lbo::cuda_fail(e, "peaks: device");
+  cudaStream_t s = (cudaStream_t)stream;
+  const int blocks = sms * lbo::kFxBlocksPerSM;
+  long long* sink = nullptr;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  e = cudaMalloc(&sink, sizeof(long long) * blocks * lbo::kFxThreads);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return LBO_ENOMEM;
+  }
+  e = cudaEventCreate(&e0);
+  if (e == cudaSuccess) e = cudaEventCreate(&e1);
+  float best = 0.f;
+  for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {  // the first warms up
+    cudaEventRecord(e0, s);
+    lbo::k_fx_transforms<<<blocks, lbo::kFxThreads, 0, s>>>(sink, kIters);
+    cudaEventRecord(e1, s);
+    e = cudaEventSynchronize(e1);
+    float ms = 0.f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    if (rep > 0 && (best == 0.f || ms < best)) best = ms;
+  }
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e0) cudaEventDestroy(e0);
+  if (e1) cudaEventDestroy(e1);
+  cudaFree(sink);
+  if (e != cudaSuccess) return lbo::cuda_fail(e, "peaks: fixed-point kernel");
+  // 5 N log2 N flops of a complex transform by convention
+  if (tflops) *tflops = 4.0 * kIters * blocks * lbo::kFxThreads * (5.0 * 32 * 5) / (best * 1e-3) / 1e12;
   return LBO_OK;
 }

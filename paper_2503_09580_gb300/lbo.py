@@ -33,7 +33,7 @@ EXPORTS = ("lbo_plan_create", "lbo_plan_set", "lbo_plan_set_stream", "lbo_apply_
            "lbo_solver_destroy", "lbo_network_param_count", "lbo_network_loss_grad", "lbo_solver_collect",
            "lbo_solver_pair_count", "lbo_solver_train_network", "lbo_solver_get_network", "lbo_solver_set_network",
            "lbo_solver_network_param_count", "lbo_plan_autotune", "lbo_group_create", "lbo_group_set_stream",
-           "lbo_group_use_graph", "lbo_group_apply_linearized", "lbo_group_destroy", "lbo_measure_alu_peaks", "lbo_plan_cache_maxwellians",
+           "lbo_group_use_graph", "lbo_group_apply_linearized", "lbo_group_destroy", "lbo_measure_alu_peaks", "lbo_measure_fx_peak", "lbo_plan_cache_maxwellians",
            "lbo_dft_axis_tensor", "lbo_evolve_homogeneous", "lbo_slab_block_transport", "lbo_slab_block_sweep",
            "lbo_slab_block_moments", "lbo_slab_cell_flux", "lbo_slab_maxwellian_cell", "lbo_vec_dots",
            "lbo_vec_axpby", "lbo_vec_combination")
@@ -144,6 +144,8 @@ def load():
     dpp = ctypes.POINTER(ctypes.c_double)
     lib.lbo_measure_alu_peaks.argtypes = [vp, dpp, dpp, ctypes.POINTER(ip), dpp]
     lib.lbo_measure_alu_peaks.restype = ip
+    lib.lbo_measure_fx_peak.argtypes = [vp, dpp]
+    lib.lbo_measure_fx_peak.restype = ip
     lib.lbo_solver_create.argtypes = [ctypes.POINTER(Problem), vp, ctypes.POINTER(vp)]
     lib.lbo_solver_create.restype = ip
     lib.lbo_newton_step.argtypes = [vp, dp, dp, ctypes.POINTER(NewtonStats)]
@@ -251,6 +253,17 @@ def measure_alu_peaks(stream=None):
     _check(lib.lbo_measure_alu_peaks(ctypes.c_void_p(stream.cuda_stream), ctypes.byref(f32), ctypes.byref(f64),
                                      ctypes.byref(sms), ctypes.byref(mhz)), "lbo_measure_alu_peaks")
     return {"fp32_tflops": f32.value, "fp64_tflops": f64.value, "sm_count": sms.value, "sm_mhz": mhz.value}
+
+
+def measure_fx_peak(stream=None):
+    """lbo_measure_fx_peak on the current device: TFLOP/s of the fixed-point
+    transforms in registers (stream as in measure_alu_peaks)."""
+    if stream is None:
+        import torch
+        stream = torch.cuda.current_stream()
+    tf = ctypes.c_double()
+    _check(load().lbo_measure_fx_peak(ctypes.c_void_p(stream.cuda_stream), ctypes.byref(tf)), "lbo_measure_fx_peak")
+    return tf.value
 
 
 class Plan:
