@@ -103,7 +103,8 @@ typedef enum {
   LBO_OPT_KERNEL = 8,      /* 0 (default): the fastest kernel set built in the
                               plan's precision (FP64, FP32X2: fixed point on the
                               integer pipe; FP32: fused at N = 32, generic at
-                              the other N, where the FP64 default is faster),
+                              the other N, where the FP64 default takes 0.1 to
+                              0.9 of its time but for L of 64 instances at N = 64),
                               1: the generic plane/axis kernels (FP64 at N = 32
                               runs the hot ones of L and of Q(f,f) with one
                               thread per pencil in registers), 2: the generic

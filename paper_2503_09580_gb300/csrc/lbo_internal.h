@@ -152,8 +152,9 @@ inline bool is_twofold_precision(int prec) { return prec == LBO_PREC_FP32X2 || p
 // FP64 and FP32X2 run in 64-bit fixed point (lin_fx.cuh, quad_fx.cuh) unless
 // LBO_OPT_KERNEL asks for other kernels.  For FP32X2 that replaces pairs of
 // FP32 numbers, which are less accurate (48 bits) and slower: L at N = 32, batch
-// 256 takes 14.2 ms in pairs against 5.7, Q at N = 64, one instance, 32.8 ms
-// against 11.0.
+// 256 takes 14.0 ms in pairs against 5.6, Q at N = 64, one instance, 32.8 ms
+// against 10.6; only Q of one radial node and one to four instances is up to 20 %
+// slower.
 inline bool uses_fixed_point(const lbo_plan* p) {
   return p->kernel_choice == 0 && (p->precision == LBO_PREC_FP64 || p->precision == LBO_PREC_FP32X2);
 }

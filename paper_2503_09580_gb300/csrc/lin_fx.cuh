@@ -18,8 +18,8 @@
 //   k_axis1_acc      InvFFT_1(sum_j phi_j FFT_1(psi^_j))
 //   k_combine_planes inverse axes 2 and 3 of L+, u and w, and L+ - u M - w g
 //
-// N = 32, 256 instances, J = 32: 5.7 ms (30.4 ms in FP64 registers, where the
-// FP64 pipe was the bound).  Arithmetic alone would take 2.3 to 2.8 ms at the
+// N = 32, 256 instances, J = 32: 5.6 ms (30.4 ms in FP64 registers, where the
+// FP64 pipe was the bound).  Arithmetic alone would take 2.0 ms at the
 // rate of register transforms, HBM 0.02 ms for inputs and outputs and about 1.5
 // for the spectra that pass between the kernels.
 //
@@ -786,8 +786,8 @@ __device__ __forceinline__ float plane_bound(float top) {
 // the time.  Two threads per pencil from N = 32 on, so that 168 registers and 12
 // warps per SM are enough: one thread per pencil took 105 us where this takes
 // 75.8 (7 instances), 16 warps of 128 registers 79.7.  A plane of 8, 16 or 32
-// threads stays within a warp and needs no block barrier.  256 instances: 2.54
-// ms, 15.2 in FP64; 5.5 TFLOP/s, 0.48 of the rate of register transforms.
+// threads stays within a warp and needs no block barrier.  256 instances: 2.51
+// ms, 15.2 in FP64; 5.55 TFLOP/s, 0.42 of the rate of register transforms.
 // grid = (N / PPC, J, B), block = Planes<N, PPC>::THREADS.
 template <int N, int PPC>
 __global__ void __launch_bounds__(Planes<N, PPC>::THREADS, Planes<N, PPC>::BLOCKS) k_plane(ci64* __restrict__ W, const int* __restrict__ EA,
@@ -1113,7 +1113,7 @@ __device__ __forceinline__ double exp2_neg64(int e) { return e > 1022 ? 0.0 : __
 // order gives the same result).  Then warp 0 transforms each column back, at
 // its own exponent EC[b][col].
 // Bound by issue and load latency; the sum over j stays on chip, where a launch
-// per node read and wrote it 32 times: 0.92 ms for 256 instances at N = 32, 4.5
+// per node read and wrote it 32 times: 0.89 ms for 256 instances at N = 32, 4.5
 // in FP64.
 // grid = (ceil(NC T / 32), B), block = 32 WARPS, shared memory acc_smem(J).
 template <int N, int WARPS>

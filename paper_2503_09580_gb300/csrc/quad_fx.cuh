@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(32) k_q_axis1(const ci64* __restrict__ R, cons
 // Bound by instruction issue: 54 % of the slots at 12 warps per SM (168
 // registers; without the bound on registers, 8 warps, 14.8 ms), its integer pipe
 // 55 %; stalls are fixed latencies and instruction fetch.  N = 32, M = 32, 32
-// instances: 13.9 ms, where the kernel that read a ready Z per node took 10.1
+// instances: 13.8 ms, where the kernel that read a ready Z per node took 10.1
 // and left 7.3 to axis 1.  The exponents of the sum belong to a row, not to the
 // plane: the largest T of a row needs a shuffle, that of a plane a barrier.
 // CARRY, from 64 nodes on: the sum's unit is 2^guard of a product's, and products
